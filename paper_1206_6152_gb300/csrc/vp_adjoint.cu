@@ -258,22 +258,15 @@ __global__ void k_force_adjoint(const double *__restrict__ lam_g, double *__rest
     lam_phi[t] = v;
 }
 
-__global__ void k_real_to_complex(const double *__restrict__ in, double2 *__restrict__ out,
-                                  long long n)
-{
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < n) out[t] = make_double2(in[t], 0.0);
-}
-
-// bc[cell] = dvol_v * lam_rho[cell], lam_rho read from the box part of the
-// real part of cbuf
-__global__ void k_bc_box(const double2 *__restrict__ cbuf, double *__restrict__ bc, int n1, int n2,
+// bc[cell] = dvol_v * lam_rho[cell], lam_rho read from the box part of
+// the FFT grid
+__global__ void k_bc_box(const double *__restrict__ lam_rho, double *__restrict__ bc, int n1, int n2,
                          int f1, int f2, double dvol_v, long long np)
 {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= np) return;
     const int k = (int)(t % n2), j = (int)((t / n2) % n1), i = (int)(t / ((long long)n1 * n2));
-    bc[t] = cbuf[((long long)i * f1 + j) * f2 + k].x * dvol_v;
+    bc[t] = lam_rho[((long long)i * f1 + j) * f2 + k] * dvol_v;
 }
 
 // lam_f[cell, v] += bc[cell]
@@ -768,14 +761,8 @@ cudaError_t launch_field_adjoint(vp_ctx *c, const double *lam_g, void *lam_f, bo
                                                            c->dx[1], c->dx[2]);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_real_to_complex<<<nblk(c->nfft, T), T, 0, c->stream>>>(lam_phi, c->cbuf, c->nfft);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    for (int a = 2; a >= 0; --a)
-        if ((e = launch_fft(c, c->cbuf, a, 0)) != cudaSuccess) return e;
-    if ((e = launch_green_mul(c)) != cudaSuccess) return e;
-    for (int a = 0; a < 3; ++a)
-        if ((e = launch_fft(c, c->cbuf, a, 1)) != cudaSuccess) return e;
-    k_bc_box<<<nblk(c->np, T), T, 0, c->stream>>>(c->cbuf, c->rho2, c->n[1], c->n[2], c->fn[1],
+    if ((e = launch_convolve(c, lam_phi, 1, lam_phi)) != cudaSuccess) return e;
+    k_bc_box<<<nblk(c->np, T), T, 0, c->stream>>>(lam_phi, c->rho2, c->n[1], c->n[2], c->fn[1],
                                                   c->fn[2], c->dvol_v, c->np);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (defer) return cudaSuccess;

@@ -54,7 +54,14 @@ __global__ void k_check(const T *__restrict__ f, long long n, unsigned long long
         if (neg) atomicAdd(cnt + 1, neg);
     }
 }
-__global__ void k_zero_lost(DevScalars *sc, double t0) { sc->lost = 0.0; sc->t = t0; sc->dt = 0.0; }
+__global__ void k_zero_lost(DevScalars *sc, double t0)
+{
+    sc->lost = 0.0;
+    sc->t = t0;
+    sc->dt = 0.0;
+    sc->amax_bits = 0;
+    sc->arrived = 0;
+}
 
 template <typename T>
 size_t coef_size() { return sizeof(LineCoef<T>); }
@@ -156,7 +163,7 @@ int build_green(vp_ctx *c)
         }
         VP_CUDA_TRY(cudaMemcpyAsync(c->cbuf, ker.data(), sizeof(double2) * nf,
                                     cudaMemcpyHostToDevice, c->stream));
-        for (int a = 2; a >= 0; --a) VP_CUDA_TRY(launch_fft(c, c->cbuf, a, 0));
+        for (int a = 2; a >= 0; --a) VP_CUDA_TRY(launch_fft(c, c->cbuf, a));
         VP_CUDA_TRY(cudaMemcpyAsync(ker.data(), c->cbuf, sizeof(double2) * nf,
                                     cudaMemcpyDeviceToHost, c->stream));
         VP_CUDA_TRY(cudaStreamSynchronize(c->stream));
@@ -223,8 +230,7 @@ int field_from_f(vp_ctx *c)
 int enqueue_prologue(vp_ctx *c)
 {
     VP_CUDA_TRY(launch_dt(c, c->g));
-    VP_CUDA_TRY(launch_coef_kick(c, c->g, &c->sc->dt, 0.5, c->coef_kick1));
-    VP_CUDA_TRY(launch_coef_drift(c, &c->sc->dt, 1.0, c->coef_drift));
+    VP_CUDA_TRY(launch_coef_step(c, c->g, c->coef_kick1, c->coef_drift));
     VP_CUDA_TRY(launch_kick(c, c->f, c->coef_kick1, nullptr, 3, 0));
     return VP_OK;
 }
@@ -252,15 +258,11 @@ int enqueue_drift_density(vp_ctx *c)
 int enqueue_body(vp_ctx *c, int last)
 {
     TRY(enqueue_drift_density(c));
-    VP_CUDA_TRY(launch_field_solve(c, c->rho, c->g));
-    VP_CUDA_TRY(launch_coef_kick(c, c->g, &c->sc->dt, 0.5, c->coef_kick2));
-    VP_CUDA_TRY(launch_advance_time(c));
+    VP_CUDA_TRY(launch_field_step(c, c->rho, c->coef_kick2, !last));
     if (last) {
         VP_CUDA_TRY(launch_kick(c, c->f, c->coef_kick2, nullptr, 3, 0));
     } else {
-        VP_CUDA_TRY(launch_dt(c, c->g));
-        VP_CUDA_TRY(launch_coef_kick(c, c->g, &c->sc->dt, 0.5, c->coef_kick1));
-        VP_CUDA_TRY(launch_coef_drift(c, &c->sc->dt, 1.0, c->coef_drift));
+        VP_CUDA_TRY(launch_coef_step(c, c->g, c->coef_kick1, c->coef_drift));
         VP_CUDA_TRY(launch_kick(c, c->f, c->coef_kick2, c->coef_kick1, 6, 0));
     }
     return VP_OK;
@@ -696,13 +698,9 @@ int vp_profile_step(vp_ctx *c, double *ms_out)
         else PROF(launch_density(c, c->f, c->rho));
         PROF(rec(4));
     }
-    PROF(launch_field_solve(c, c->rho, c->g));
+    PROF(launch_field_step(c, c->rho, c->coef_kick2, 1));
     PROF(rec(5));
-    PROF(launch_coef_kick(c, c->g, &c->sc->dt, 0.5, c->coef_kick2));
-    PROF(launch_advance_time(c));
-    PROF(launch_dt(c, c->g));
-    PROF(launch_coef_kick(c, c->g, &c->sc->dt, 0.5, c->coef_kick1));
-    PROF(launch_coef_drift(c, &c->sc->dt, 1.0, c->coef_drift));
+    PROF(launch_coef_step(c, c->g, c->coef_kick1, c->coef_drift));
     PROF(rec(6));
     if (big_kick) c->kick_pass_ev = ev + 8;
     {

@@ -163,6 +163,17 @@ __device__ __forceinline__ double block_max(double v, double *scratch)
     return v;
 }
 
+// x / 6, correctly rounded for normal x and quotient: the quotient by the
+// rounded reciprocal and one residual correction (Brisebarre, Muller & Raina,
+// "Accelerating correctly rounded floating-point division when the divisor is
+// known in advance", 2004).  Three FP64 instructions, 64 cycles of the FP64
+// pipe each per warp, where a division takes about three times as many.
+__device__ __forceinline__ double div6(double x)
+{
+    const double z = 1.0 / 6.0, q = x * z;
+    return fma(fma(-6.0, q, x), z, q);
+}
+
 // Shift alpha = u tau / h as LineCoef (FP64 in, the storage type out).
 template <typename T>
 __device__ __forceinline__ LineCoef<T> make_line_coef(double alpha)
@@ -175,7 +186,7 @@ __device__ __forceinline__ LineCoef<T> make_line_coef(double alpha)
     const double b = a - s;
     c.code = 2 * (int)s + neg;
     c.c0 = (T)b;
-    c.c1 = (T)(b * (1.0 - b) * (2.0 - b) / 6.0);
-    c.c2 = (T)(b * (1.0 - b) * (1.0 + b) / 6.0);
+    c.c1 = (T)div6(b * (1.0 - b) * (2.0 - b));
+    c.c2 = (T)div6(b * (1.0 - b) * (1.0 + b));
     return c;
 }

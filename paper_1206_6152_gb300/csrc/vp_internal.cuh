@@ -35,6 +35,15 @@ struct DevScalars {
     double lost;        // phase-space sum of f that left (unscaled)
     double amax;        // max_l,x |g_l| / dv_l of the last dt evaluation
     double pad[6];      // per-call scalars of the entry points (stream-ordered)
+    unsigned long long amax_bits;   // running maximum of a dt evaluation (0 between launches)
+    unsigned int arrived;           // CTAs that have added theirs (0 between launches)
+};
+
+// dt = C min(dt_p, dt_v) (Sec. 2.4): 1/dv per axis, dt_p, the Courant number,
+// a fixed dt (> 0); advance: t += the old dt first
+struct DtParams {
+    double idv0, idv1, idv2, dtp, courant, dt_fixed;
+    int advance;
 };
 
 struct FFTAxis {
@@ -111,8 +120,9 @@ struct vp_ctx {
 cudaError_t launch_coef_drift(vp_ctx *c, const double *tau_ptr, double factor, void *out);
 cudaError_t launch_coef_kick(vp_ctx *c, const double *g, const double *tau_ptr, double factor,
                              void *out);
+// the tables of a step from sc->dt: first half kick (dt / 2) of g, drifts (dt)
+cudaError_t launch_coef_step(vp_ctx *c, const double *g, void *kick, void *drift);
 cudaError_t launch_dt(vp_ctx *c, const double *g);
-cudaError_t launch_advance_time(vp_ctx *c);
 // drift along a spatial axis; max_alpha is a host-side bound of |v tau / dx|
 // over the table (the register kernels need it below 1); with rho_part the
 // x drift also writes density partials (returns cudaErrorNotSupported if it
@@ -125,6 +135,11 @@ cudaError_t launch_kick(vp_ctx *c, void *f, const void *coef_a, const void *coef
                         int first_axis);
 cudaError_t launch_density(vp_ctx *c, const void *f, double *rho);
 cudaError_t launch_field_solve(vp_ctx *c, const double *rho, double *g_out);
+// the field of the step: phi and c->g of rho, the second half kick's table, t
+// += dt and, with next, the dt of the next step
+cudaError_t launch_field_step(vp_ctx *c, const double *rho, void *kick, int next);
+// out = G * in on the FFT grid (real); whole: in covers it, else the box
+cudaError_t launch_convolve(vp_ctx *c, const double *in, int whole, double *out);
 cudaError_t launch_energy_partials(vp_ctx *c, const void *f, double *partials);
 cudaError_t launch_copy_phi_box(vp_ctx *c, double *dst);
 cudaError_t launch_dot_rho_phi(vp_ctx *c, const double *rho, double *out2);
@@ -170,9 +185,8 @@ cudaError_t launch_sweep_into(vp_ctx *c, const void *src, void *dst, int axis, c
 cudaError_t launch_rho_finish(vp_ctx *c, const double *part, int nparts, double *rho);
 
 int vp_fft_plan_axis(FFTAxis *a, int n);
-cudaError_t launch_fft(vp_ctx *c, double2 *data, int axis, int inverse);
+cudaError_t launch_fft(vp_ctx *c, double2 *data, int axis);
 
-cudaError_t launch_green_mul(vp_ctx *c);
 double vp_drift_alpha_bound(const vp_ctx *c, double tau);
 
 // adjoint (vp_adjoint.cu)

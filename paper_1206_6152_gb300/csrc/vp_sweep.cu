@@ -337,30 +337,32 @@ __global__ void k_coef_kick(LineCoef<T> *out, const double *__restrict__ g, long
     out[t] = make_line_coef<T>(g[a * np + cell] * tau / dv);
 }
 
-// dt = C min(dt_p, dt_v) (Sec. 2.4), or the fixed dt.  One CTA.
-__global__ void k_dt(DevScalars *sc, const double *__restrict__ g, long long np, double idv0,
-                     double idv1, double idv2, double dtp, double courant, double dt_fixed)
+// both tables of a step from sc->dt, one launch: [0, 3 np) the first half
+// kick's (dt / 2), then the drifts' (dt)
+template <typename T>
+__global__ void k_coef_step(LineCoef<T> *__restrict__ kick, const double *__restrict__ g,
+                            long long np, double dv0, double dv1, double dv2,
+                            LineCoef<T> *__restrict__ drift, int maxnv, int nv0, int nv1, int nv2,
+                            const double *vc0, const double *vc1, const double *vc2, double dx0,
+                            double dx1, double dx2, const DevScalars *sc)
 {
-    __shared__ double red[32];
-    double m = 0.0;
-    for (long long i = threadIdx.x; i < np; i += blockDim.x) {
-        m = fmax(m, fabs(g[i]) * idv0);
-        m = fmax(m, fabs(g[np + i]) * idv1);
-        m = fmax(m, fabs(g[2 * np + i]) * idv2);
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < 3 * np) {
+        const long long cell = t / 3;
+        const int a = (int)(t - cell * 3);
+        const double dv = a == 0 ? dv0 : (a == 1 ? dv1 : dv2);
+        const double tau = sc->dt * 0.5;
+        kick[t] = make_line_coef<T>(g[a * np + cell] * tau / dv);
+        return;
     }
-    m = block_max(m, red);
-    if (threadIdx.x == 0) {
-        sc->amax = m;
-        if (dt_fixed > 0.0) {
-            sc->dt = dt_fixed;
-        } else {
-            const double dtv = m > 0.0 ? 1.0 / m : INFINITY;
-            sc->dt = courant * fmin(dtp, dtv);
-        }
-    }
+    const int u = (int)(t - 3 * np), a = u / maxnv, j = u - a * maxnv;
+    if (a >= 3) return;
+    const int nva = a == 0 ? nv0 : (a == 1 ? nv1 : nv2);
+    if (j >= nva) return;
+    const double *vc = a == 0 ? vc0 : (a == 1 ? vc1 : vc2);
+    const double dx = a == 0 ? dx0 : (a == 1 ? dx1 : dx2);
+    drift[u] = make_line_coef<T>(vc[j] * sc->dt / dx);
 }
-
-__global__ void k_advance_time(DevScalars *sc) { sc->t += sc->dt; }
 
 // ---------------------------------------------------------------------------
 // rho(x) = dv^3 sum_v f (Sec. 2.2): one CTA per velocity cube, compensated
@@ -607,22 +609,21 @@ cudaError_t launch_coef_kick(vp_ctx *c, const double *g, const double *tau_ptr, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_dt(vp_ctx *c, const double *g)
+template <typename T>
+static cudaError_t coef_step_t(vp_ctx *c, const double *g, LineCoef<T> *kick, LineCoef<T> *drift)
 {
-    double dtp = INFINITY;
-    for (int a = 0; a < 3; ++a) {
-        const double vmax = fmax(fabs(c->cfg.vlo[a]), fabs(c->cfg.vhi[a]));
-        if (vmax > 0) dtp = fmin(dtp, c->dx[a] / vmax);
-    }
-    k_dt<<<1, 1024, 0, c->stream>>>(c->sc, g, c->np, 1.0 / c->dv[0], 1.0 / c->dv[1],
-                                    1.0 / c->dv[2], dtp, c->cfg.courant, c->cfg.dt_fixed);
+    const long long total = 3 * c->np + 3 * c->maxnv;
+    k_coef_step<T><<<(unsigned)((total + 63) / 64), 64, 0, c->stream>>>(
+        kick, g, c->np, c->dv[0], c->dv[1], c->dv[2], drift, c->maxnv, c->nv[0], c->nv[1], c->nv[2],
+        c->vc[0], c->vc[1], c->vc[2], c->dx[0], c->dx[1], c->dx[2], c->sc);
     return cudaGetLastError();
 }
 
-cudaError_t launch_advance_time(vp_ctx *c)
+cudaError_t launch_coef_step(vp_ctx *c, const double *g, void *kick, void *drift)
 {
-    k_advance_time<<<1, 1, 0, c->stream>>>(c->sc);
-    return cudaGetLastError();
+    if (c->isdouble)
+        return coef_step_t<double>(c, g, (LineCoef<double> *)kick, (LineCoef<double> *)drift);
+    return coef_step_t<float>(c, g, (LineCoef<float> *)kick, (LineCoef<float> *)drift);
 }
 
 cudaError_t launch_drift(vp_ctx *c, void *f, int axis, const void *coef, double max_alpha,
