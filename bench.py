@@ -408,7 +408,7 @@ def record_traffic(csv_path, workload):
         elif "k_kick_pass_c" in name: slot = "kick_c"
         elif "k_kick6" in name: slot = "kick6"
         elif "k_drift_yz" in name: slot = "drift_yz"
-        elif "k_drift_fast" in name and name.replace(" ", "").split(",")[3].startswith("1>"):
+        elif "k_drift_fast" in name and name.split("k_drift_fast<")[1].split(">")[0].split(",")[-1].strip() == "1":
             slot = "drift_x"
         elif "k_drift_fast" in name:
             slot = ("drift_z", "drift_y")[zy % 2]

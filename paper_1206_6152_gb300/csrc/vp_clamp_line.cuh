@@ -1,0 +1,94 @@
+// vp_clamp_line.cuh -- the PFC update of one line of run-time length held in
+// registers, in the clamp form of the slope corrector (pfc_flux of
+// vp_device.cuh, bit for bit), for lines of any length up to a compile-time
+// NMAX.
+//
+// The line is held in upwind order: a line with u < 0 is read and written from
+// its far end with a negative stride, so that the lanes of a warp run one code
+// path whatever their directions (a z drift has both signs of v_z in every
+// warp).  x[n .. NMAX] hold what lies beyond the line's end: its first cell
+// (periodic) or 0 (outflow).
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "vp_device.cuh"
+
+namespace vpline {
+
+// 2 a and -a.  FP64: on the integer pipes (an FP64 instruction, a negation or
+// one that is predicated off included, takes 64 cycles of a quadrant's FP64
+// pipe): 2 a is the exponent plus one, for zeros and subnormals the mantissa
+// shifted, for infinities and NaN a itself, infinity where it overflows.
+__device__ __forceinline__ float twice(float a) { return a + a; }
+__device__ __forceinline__ double twice(double a)
+{
+    const unsigned hi = (unsigned)__double2hiint(a), lo = (unsigned)__double2loint(a);
+    const unsigned e = hi & 0x7ff00000u, s = hi & 0x80000000u;
+    unsigned h2 = e ? hi + 0x00100000u : s | (((hi << 1) | (lo >> 31)) & 0x7fffffffu);
+    unsigned l2 = e ? lo : lo << 1;
+    if (e >= 0x7fe00000u) {
+        h2 = e == 0x7ff00000u ? hi : (s | 0x7ff00000u);
+        l2 = e == 0x7ff00000u ? lo : 0u;
+    }
+    return __hiloint2double((int)h2, (int)l2);
+}
+__device__ __forceinline__ float negate(float a) { return -a; }
+__device__ __forceinline__ double negate(double a)
+{
+    return __hiloint2double(__double2hiint(a) ^ (int)0x80000000, __double2loint(a));
+}
+
+// pfc_flux with the differences dp = fp - f0 and dm = f0 - fm (each cell's dp
+// is the next one's dm).  FP64: with the difference and the two additions of
+// the update 7 FP64 instructions per cell.
+template <typename T>
+__device__ __forceinline__ T clamp_flux(T dm, T f0, T dp, T finf, T c0, T c1, T c2)
+{
+    const T a = twice(f0), b = twice(finf - f0);
+    const T ep = vmin(vmax(dp, negate(b)), a);
+    const T em = vmin(vmax(dm, negate(a)), b);
+    const T phi = c0 * f0 + c1 * ep + c2 * em;
+    return vmin(vmax(phi, T(0)), f0);
+}
+
+// maximum of the line and 0
+template <typename T, int NMAX>
+__device__ __forceinline__ T clamp_line_max(const T (&x)[NMAX + 1], int n)
+{
+    T m = T(0);
+#pragma unroll
+    for (int j = 0; j < NMAX; ++j) {
+        if (j >= n) break;
+        m = vmax(m, x[j]);
+    }
+    return m;
+}
+
+// the zero-shift update of the line x; put(j, v) takes cell j's new value, in
+// increasing j, after every cell of the line has been read.  PERIODIC: fm1,
+// fm2 are the line's last and last but one cells.  Returns the last cell's
+// flux (what leaves an outflow line).
+template <typename T, int NMAX, bool PERIODIC, class P>
+__device__ __forceinline__ T clamp_line(const T (&x)[NMAX + 1], int n, T fm1, T fm2, T c0, T c1, T c2,
+                                        P put)
+{
+    const T finf = clamp_line_max<T, NMAX>(x, n);
+    T dm = x[0], phm = T(0);                    // outflow: f_{-1} = 0
+    if (PERIODIC) {
+        dm = x[0] - fm1;
+        phm = clamp_flux(fm1 - fm2, fm1, dm, finf, c0, c1, c2);
+    }
+#pragma unroll
+    for (int j = 0; j < NMAX; ++j) {
+        if (j >= n) break;          // a branch: cells past the end take no issue slots
+        const T dp = x[j + 1] - x[j];
+        const T ph = clamp_flux(dm, x[j], dp, finf, c0, c1, c2);
+        put(j, (x[j] - ph) + phm);
+        phm = ph;
+        dm = dp;
+    }
+    return phm;
+}
+
+}  // namespace vpline

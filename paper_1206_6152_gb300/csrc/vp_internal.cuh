@@ -178,6 +178,10 @@ cudaError_t launch_kick_fast(vp_ctx *c, void *f, const void *ca, const void *cb,
                              void *inter1 = nullptr, const int *gate = nullptr);
 cudaError_t launch_drift_fast(vp_ctx *c, void *f, int axis, const void *coef, double *rho_part,
                               void *fo = nullptr);
+// sweeps of lines of any length up to 64, zero shift (vp_sweep_lines.cu); f
+// into fo (fo == f: in place)
+int vp_drift_lines_ok(const vp_ctx *c, int axis);
+cudaError_t launch_drift_lines(vp_ctx *c, const void *f, int axis, const void *coef, void *fo);
 // one sweep from src into dst (dst != src), used by the adjoint's replay;
 // kick tables [np][3], drift tables [3][maxnv]
 cudaError_t launch_sweep_into(vp_ctx *c, const void *src, void *dst, int axis, const void *coef,

@@ -632,6 +632,7 @@ cudaError_t launch_drift(vp_ctx *c, void *f, int axis, const void *coef, double 
     const bool fast = vp_drift_fast_ok(c, axis) && max_alpha < 1.0;
     if (rho_part && !(fast && axis == 0 && vp_rho_fuse_ok(c))) return cudaErrorNotSupported;
     if (fast) return launch_drift_fast(c, f, axis, coef, rho_part);
+    if (vp_drift_lines_ok(c, axis) && max_alpha < 1.0) return launch_drift_lines(c, f, axis, coef, f);
     if (c->isdouble)
         return launch_drift_t<double>(c, (double *)f, axis, (const LineCoef<double> *)coef);
     return launch_drift_t<float>(c, (float *)f, axis, (const LineCoef<float> *)coef);
@@ -662,6 +663,8 @@ cudaError_t launch_sweep_into(vp_ctx *c, const void *src, void *dst, int axis, c
         return launch_kick_f64(c, const_cast<void *>(src), coef, nullptr, 1, axis - 3, dst);
     if (axis < 3 && vp_drift_fast_ok(c, axis) && drift_alpha_bound < 1.0)
         return launch_drift_fast(c, const_cast<void *>(src), axis, coef, nullptr, dst);
+    if (axis < 3 && vp_drift_lines_ok(c, axis) && drift_alpha_bound < 1.0)
+        return launch_drift_lines(c, src, axis, coef, dst);
     cudaError_t e = cudaMemcpyAsync(dst, src, (size_t)c->ncells * c->esize,
                                     cudaMemcpyDeviceToDevice, c->stream);
     if (e != cudaSuccess) return e;

@@ -9,10 +9,9 @@
 //    f32x2 arithmetic; vz sweep: one contiguous line per thread with 16-byte
 //    shared loads.  A cube-sweep whose shift has a whole-cell part falls back
 //    to the generic in-place line routine.
-//  * k_drift_fast<T, N>: each thread owns two (float) or one (double)
-//    position lines, loads them straight from global memory into registers
-//    (a warp reads 256 contiguous bytes per load), updates them and stores
-//    them back.  Optionally (x sweep) it accumulates the density of the
+//  * k_drift_fast<N>: each thread owns two position lines, loads them straight
+//    from global memory into registers (a warp reads 256 contiguous bytes per
+//    load), updates them and stores them back.  Optionally (x sweep) it accumulates the density of the
 //    updated f: per-thread double-float sums over the velocity cells it
 //    visits (kept in the thread's shared-memory slots), one reduction per
 //    CTA into a small partial buffer.
@@ -501,17 +500,10 @@ struct DriftGeom {
     long long np;
 };
 
-template <typename T>
-struct DriftVec;
-template <>
-struct DriftVec<float> { typedef float2 V; static constexpr int W = 2; };
-template <>
-struct DriftVec<double> { typedef double V; static constexpr int W = 1; };
-
 // logical unit index -> first velocity cell of the unit
-__device__ __forceinline__ long long unit_to_v(long long L, const DriftGeom &g, int W)
+__device__ __forceinline__ long long unit_to_v(long long L, const DriftGeom &g)
 {
-    if (W == 2 && g.zremap > 0) {
+    if (g.zremap > 0) {
         const int H = g.zremap;           // pairs per half row
         const int RW = 32 / H;            // rows per warp
         const long long q = L % H;
@@ -523,88 +515,62 @@ __device__ __forceinline__ long long unit_to_v(long long L, const DriftGeom &g, 
         const long long row = rg * RW + ri;
         return row * g.nvz + (h * H + q) * 2;
     }
-    return L * W;
+    return L * 2;
 }
 
 // RHO: the per-thread compensated density sums of the N cells of the line
 // live in shared memory (slot j of thread t at j * 128 + t: conflict-free),
 // which keeps the kernel at 128 registers (16 warps per SM)
-template <typename T, int N, bool PERIODIC, bool RHO>
-__global__ void __launch_bounds__(128, N <= 32 ? 4 : 1) k_drift_fast(const T *__restrict__ f,
-                                                               const LineCoef<T> *__restrict__ coef,
+template <int N, bool PERIODIC, bool RHO>
+__global__ void __launch_bounds__(128, N <= 32 ? 4 : 1) k_drift_fast(const float *__restrict__ f,
+                                                               const LineCoef<float> *__restrict__ coef,
                                                                DriftGeom g, double *__restrict__ rho_part,
-                                                               double *lost_out, T *__restrict__ fo)
+                                                               double *lost_out, float *__restrict__ fo)
 {
-    typedef typename DriftVec<T>::V V;
-    constexpr int W = DriftVec<T>::W;
     __shared__ Acc<double> red[32];
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    Acc<T> *sacc = reinterpret_cast<Acc<T> *>(smem_raw) + threadIdx.x;   // slot j: sacc[j * 128]
+    Acc<float> *sacc = reinterpret_cast<Acc<float> *>(smem_raw) + threadIdx.x;   // slot j: sacc[j * 128]
     const int o = blockIdx.y;
     const long long base_cell = (long long)(o / g.od) * g.m1 + (long long)(o % g.od) * g.m2;
     const long long gstride = g.cell_stride * g.nvc;
-    const T *fb = f + base_cell * g.nvc;
-    T *ob = fo + base_cell * g.nvc;
+    const float *fb = f + base_cell * g.nvc;
+    float *ob = fo + base_cell * g.nvc;
     const long long u0 = (long long)blockIdx.x * g.per_part;
     long long u1 = u0 + g.per_part;
     if (u1 > g.nunits) u1 = g.nunits;
     if constexpr (RHO) {
 #pragma unroll
-        for (int j = 0; j < N; ++j) sacc[j * 128] = Acc<T>();
+        for (int j = 0; j < N; ++j) sacc[j * 128] = Acc<float>();
     }
-    T lost = T(0);
+    float lost = 0.f;
     for (long long L = u0 + threadIdx.x; L < u1; L += blockDim.x) {
-        const long long v = unit_to_v(L, g, W);
-        V x[N];
+        const long long v = unit_to_v(L, g);
+        float2 x[N];
         // the line's addresses are stepped through an opaque register: the
         // compiler would otherwise keep all 2 N of them live across the update
-        const T *p = fb + v;
+        const float *p = fb + v;
 #pragma unroll
         for (int j = 0; j < N; ++j) {
-            x[j] = *reinterpret_cast<const V *>(p);
+            x[j] = *reinterpret_cast<const float2 *>(p);
             p += gstride;
             asm volatile("" : "+l"(p));
         }
-        if constexpr (W == 2) {
-            const int via = (int)((v / g.va_stride) % g.va_n);
-            const int vib = (int)(((v + 1) / g.va_stride) % g.va_n);
-            const LineCoef<float> ca = coef[via];
-            const LineCoef<float> cb = coef[vib];
-            if ((ca.code & 1) == (cb.code & 1)) {
-                const LineW<float2> w = weights_pair2(ca, cb, line_max(x));
-                const float2 out = update_line<float2, N, PERIODIC>(x, w, ca.code & 1);
-                lost += out.x + out.y;
-            } else {
-                // the pair straddles the sign change of the velocity: two
-                // scalar lines
-                float y0[N], y1[N];
-#pragma unroll
-                for (int j = 0; j < N; ++j) { y0[j] = x[j].x; y1[j] = x[j].y; }
-                const LineW<float> w0 = weights_one<float>(ca, line_max(y0));
-                const LineW<float> w1 = weights_one<float>(cb, line_max(y1));
-                lost += update_line<float, N, PERIODIC>(y0, w0, ca.code & 1);
-                lost += update_line<float, N, PERIODIC>(y1, w1, cb.code & 1);
-#pragma unroll
-                for (int j = 0; j < N; ++j) x[j] = make_float2(y0[j], y1[j]);
-            }
-        } else {
-            const int via = (int)((v / g.va_stride) % g.va_n);
-            const LineCoef<T> ca = coef[via];
-            lost += update_line_f64<N, PERIODIC>(x, ca.c0, ca.c1, ca.c2, ca.code & 1);
-        }
-        T *q = ob + v;
+        const int via = (int)((v / g.va_stride) % g.va_n);
+        const int vib = (int)(((v + 1) / g.va_stride) % g.va_n);
+        lost += drift_pair<N, PERIODIC>(x, coef[via], coef[vib]);
+        float *q = ob + v;
 #pragma unroll
         for (int j = 0; j < N; ++j) {
-            *reinterpret_cast<V *>(q) = x[j];
+            *reinterpret_cast<float2 *>(q) = x[j];
             q += gstride;
             asm volatile("" : "+l"(q));
         }
         if constexpr (RHO) {
 #pragma unroll
             for (int j = 0; j < N; ++j) {
-                Acc<T> a = sacc[j * 128];
-                if constexpr (W == 2) { a.add(x[j].x); a.add(x[j].y); }
-                else a.add(x[j]);
+                Acc<float> a = sacc[j * 128];
+                a.add(x[j].x);
+                a.add(x[j].y);
                 sacc[j * 128] = a;
             }
         }
@@ -613,7 +579,7 @@ __global__ void __launch_bounds__(128, N <= 32 ? 4 : 1) k_drift_fast(const T *__
         // per-x reduction over the CTA, written as one partial per (part, cell)
 #pragma unroll
         for (int j = 0; j < N; ++j) {
-            Acc<T> a = block_merge(sacc[j * 128], reinterpret_cast<Acc<T> *>(red));
+            Acc<float> a = block_merge(sacc[j * 128], reinterpret_cast<Acc<float> *>(red));
             if (threadIdx.x == 0)
                 rho_part[(long long)blockIdx.x * g.np + base_cell + j * g.cell_stride] = a.value();
             __syncthreads();
@@ -801,9 +767,9 @@ cudaError_t kick_fast_n(vp_ctx *c, float *f, const LineCoef<float> *ca, const Li
     return cudaGetLastError();
 }
 
-template <typename T, int N>
-cudaError_t drift_fast_n(vp_ctx *c, T *f, int axis, const LineCoef<T> *coef, double *rho_part,
-                         int nparts, T *fo)
+template <int N>
+cudaError_t drift_fast_n(vp_ctx *c, float *f, int axis, const LineCoef<float> *coef, double *rho_part,
+                         int nparts, float *fo)
 {
     DriftGeom g;
     if (axis == 0) {
@@ -816,15 +782,14 @@ cudaError_t drift_fast_n(vp_ctx *c, T *f, int axis, const LineCoef<T> *coef, dou
         g.cell_stride = 1;
         g.od = 1; g.m1 = c->n[2]; g.m2 = 0;
     }
-    constexpr int W = DriftVec<T>::W;
     g.nvc = c->nvc;
     g.va_stride = axis == 0 ? c->nv[1] * c->nv[2] : (axis == 1 ? c->nv[2] : 1);
     g.va_n = c->nv[axis];
-    g.nunits = c->nvc / W;
+    g.nunits = c->nvc / 2;
     g.nvz = c->nv[2];
     g.np = c->np;
     g.zremap = 0;
-    if (W == 2 && axis == 2 && c->nv[2] % 4 == 0) {
+    if (axis == 2 && c->nv[2] % 4 == 0) {
         const int H = c->nv[2] / 4;
         if (32 % H == 0 && ((long long)c->nv[0] * c->nv[1]) % (2 * (32 / H)) == 0) g.zremap = H;
     }
@@ -838,33 +803,17 @@ cudaError_t drift_fast_n(vp_ctx *c, T *f, int axis, const LineCoef<T> *coef, dou
     }
     g.per_part = (g.nunits + nparts - 1) / nparts;
     dim3 grid((unsigned)nparts, (unsigned)outer);
-    const bool rho = rho_part != nullptr;
-    constexpr bool RHO_OK = (sizeof(T) == 4 && N <= 64) || N <= 16;
-    if (rho && !RHO_OK) return cudaErrorNotSupported;
-    constexpr size_t racc = (size_t)N * 128 * sizeof(Acc<T>);   // density sums (RHO)
-    if constexpr (RHO_OK) {
-        if (rho) {
-            cudaError_t e = cudaFuncSetAttribute(c->periodic_space ? k_drift_fast<T, N, true, true>
-                                                                   : k_drift_fast<T, N, false, true>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)racc);
-            if (e != cudaSuccess) return e;
-        }
-    }
-    if (c->periodic_space) {
-        if constexpr (RHO_OK)
-            if (rho) {
-                k_drift_fast<T, N, true, true><<<grid, 128, racc, c->stream>>>(f, coef, g, rho_part, &c->sc->lost, fo ? fo : f);
-                return cudaGetLastError();
-            }
-        k_drift_fast<T, N, true, false><<<grid, 128, 0, c->stream>>>(f, coef, g, rho_part, &c->sc->lost, fo ? fo : f);
+    float *o = fo ? fo : f;
+    double *lost = &c->sc->lost;
+    if (rho_part) {
+        constexpr size_t racc = (size_t)N * 128 * sizeof(Acc<float>);   // density sums
+        auto kern = c->periodic_space ? k_drift_fast<N, true, true> : k_drift_fast<N, false, true>;
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)racc);
+        if (e != cudaSuccess) return e;
+        kern<<<grid, 128, racc, c->stream>>>(f, coef, g, rho_part, lost, o);
     } else {
-        if constexpr (RHO_OK)
-            if (rho) {
-                k_drift_fast<T, N, false, true><<<grid, 128, racc, c->stream>>>(f, coef, g, rho_part, &c->sc->lost, fo ? fo : f);
-                return cudaGetLastError();
-            }
-        k_drift_fast<T, N, false, false><<<grid, 128, 0, c->stream>>>(f, coef, g, rho_part, &c->sc->lost, fo ? fo : f);
+        auto kern = c->periodic_space ? k_drift_fast<N, true, false> : k_drift_fast<N, false, false>;
+        kern<<<grid, 128, 0, c->stream>>>(f, coef, g, rho_part, lost, o);
     }
     return cudaGetLastError();
 }
@@ -878,7 +827,7 @@ int vp_rho_parts(vp_ctx *c)
     long long target = 4LL * 4 * vp_sm_count();
     int nparts = (int)((target + outer - 1) / outer);
     if (nparts < 1) nparts = 1;
-    const long long nunits = c->nvc / (c->isdouble ? 1 : 2);
+    const long long nunits = c->nvc / 2;
     const long long maxparts = (nunits + 127) / 128;
     if (nparts > maxparts) nparts = (int)maxparts;
     return nparts;
@@ -894,15 +843,12 @@ int vp_kick_fast_ok(const vp_ctx *c)
 int vp_drift_fast_ok(const vp_ctx *c, int axis)
 {
     const int n = c->n[axis];
-    if (!(n == 16 || n == 32 || n == 48 || n == 64)) return 0;
-    if (!c->isdouble && (c->nvc % 2 != 0)) return 0;
-    if (c->isdouble && n > 32) return 0;
-    return 1;
+    return !c->isdouble && c->nvc % 2 == 0 && (n == 16 || n == 32 || n == 48 || n == 64);
 }
 
 int vp_rho_fuse_ok(const vp_ctx *c)
 {
-    return vp_drift_fast_ok(c, 0) && c->n[0] <= (c->isdouble ? 16 : 64);
+    return vp_drift_fast_ok(c, 0);
 }
 
 cudaError_t launch_kick_fast(vp_ctx *c, void *f, const void *ca, const void *cb, int nsweeps,
@@ -921,18 +867,13 @@ cudaError_t launch_drift_fast(vp_ctx *c, void *f, int axis, const void *coef, do
 {
     const int n = c->n[axis];
     const int np = rho_part ? vp_rho_parts(c) : 0;
-    if (c->isdouble) {
-        const LineCoef<double> *cf = (const LineCoef<double> *)coef + (size_t)axis * c->maxnv;
-        if (n == 32) return drift_fast_n<double, 32>(c, (double *)f, axis, cf, rho_part, np, (double *)fo);
-        return drift_fast_n<double, 16>(c, (double *)f, axis, cf, rho_part, np, (double *)fo);
-    }
     const LineCoef<float> *cf = (const LineCoef<float> *)coef + (size_t)axis * c->maxnv;
     float *o = (float *)fo;
     switch (n) {
-    case 16: return drift_fast_n<float, 16>(c, (float *)f, axis, cf, rho_part, np, o);
-    case 32: return drift_fast_n<float, 32>(c, (float *)f, axis, cf, rho_part, np, o);
-    case 48: return drift_fast_n<float, 48>(c, (float *)f, axis, cf, rho_part, np, o);
-    default: return drift_fast_n<float, 64>(c, (float *)f, axis, cf, rho_part, np, o);
+    case 16: return drift_fast_n<16>(c, (float *)f, axis, cf, rho_part, np, o);
+    case 32: return drift_fast_n<32>(c, (float *)f, axis, cf, rho_part, np, o);
+    case 48: return drift_fast_n<48>(c, (float *)f, axis, cf, rho_part, np, o);
+    default: return drift_fast_n<64>(c, (float *)f, axis, cf, rho_part, np, o);
     }
 }
 

@@ -1,0 +1,66 @@
+"""Sweeps of lines of any length (one line per thread in registers) against the
+FP64 oracle at the lengths where those kernels can go wrong: one and two cells,
+the last length of each register size and the first of the next, the longest
+they take and one beyond (the shared-memory kernels), lines of both directions
+in a warp, last CTAs that are not full, both boundary rules, and shifts of a
+cell or more beside sub-cell ones."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytestmark = pytest.mark.skip(reason="needs a CUDA GPU")
+
+from oracle import vp_oracle as O  # noqa: E402
+from paper_1206_6152_gb300 import inputs as I  # noqa: E402
+
+DEV = "cuda:0"
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_1206_6152_gb300 import build as B
+    B.build()
+
+
+def compare_sweep(w, axis, taus, seed):
+    """One sweep per tau against the oracle; f has zeros and a wide range."""
+    from paper_1206_6152_gb300.vlasov import VlasovPoisson, config_of
+    rng = np.random.default_rng(seed)
+    np_t = np.float32 if w.dtype == "f32" else np.float64
+    f0 = (rng.random(w.shape) * np.exp(-8 * rng.random(w.shape)) * (rng.random(w.shape) > 0.1)).astype(np_t)
+    acc = rng.normal(size=(3,) + w.n)
+    grid, per = O.Grid.of(w), w.space_bc == "periodic"
+    f = torch.from_numpy(f0).to(DEV)
+    with VlasovPoisson(config_of(w), f) as sim:
+        sim.set_accel(torch.from_numpy(acc))
+        for tau in taus:
+            f.copy_(torch.from_numpy(f0))
+            lost0 = sim.energy()["M_out"]
+            sim.sweep(axis, tau)
+            ref = f0.astype(np.float64)
+            if axis < 3:
+                lost = O.sweep(ref, axis, grid.vc(axis), tau, grid.dx[axis], per)
+            else:
+                lost = O.sweep(ref, axis, acc[axis - 3], tau, grid.dv[axis - 3], False)
+            got = f.cpu().numpy().astype(np.float64)
+            # one rounding of each flux and update in the storage type
+            tol = 1e-12 if w.dtype == "f64" else 2e-6
+            assert np.abs(got - ref).max() <= tol * f0.max(), (axis, tau)
+            assert got.min() >= 0.0
+            lost_g = (sim.energy()["M_out"] - lost0) / (grid.dvol_x * grid.dvol_v)
+            assert abs(lost_g - lost) <= 50 * tol * max(lost, f0.sum() * 1e-3), (axis, tau)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("space_bc", ["periodic", "outflow"])
+@pytest.mark.parametrize("n", [1, 2, 15, 18, 33, 63, 65])
+def test_drift_lines_match_oracle(n, space_bc, dtype):
+    for axis in range(3):
+        shape = [2, 3, 2]
+        shape[axis] = n
+        nv = (5, 7, 6)                  # 210 velocity cells: the last CTA is not full
+        w = I.small_maxwell(n=tuple(shape), nv=nv, dtype=dtype, space_bc=space_bc)
+        h, v = w.dx[axis], max(abs(w.vlo[axis]), abs(w.vhi[axis]))
+        compare_sweep(w, axis, (0.7 * h / v, -0.97 * h / v, 2.3 * h / v), 10 * n + axis)
