@@ -88,13 +88,19 @@ struct Acc<float> {
 template <>
 struct Acc<double> {
     double s = 0.0, c = 0.0;
+    // Neumaier's sum with the larger operand chosen by its exponent (that is
+    // all the error term needs to be exact) on the integer pipes: four FP64
+    // instructions of 74 pipe cycles each; comparing and subtracting in both
+    // orders took eight
     __device__ __forceinline__ void add(double x)
     {
         const double t = s + x;
-        if (fabs(s) >= fabs(x))
-            c += (s - t) + x;
-        else
-            c += (x - t) + s;
+        const int sh = __double2hiint(s), sl = __double2loint(s);
+        const int xh = __double2hiint(x), xl = __double2loint(x);
+        const bool ge = (sh & 0x7fffffff) >= (xh & 0x7fffffff);
+        const double big = __hiloint2double(ge ? sh : xh, ge ? sl : xl);
+        const double small = __hiloint2double(ge ? xh : sh, ge ? xl : sl);
+        c += (big - t) + small;
         s = t;
     }
     __device__ __forceinline__ void merge(const Acc<double> &o)

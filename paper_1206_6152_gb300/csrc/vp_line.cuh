@@ -29,7 +29,7 @@ namespace vpline {
 
 // ---------------------------------------------------------------------------
 // small vector abstraction: float2 (two lines packed, f32x2 instructions) or
-// a scalar float/double (one line)
+// a scalar float (one line)
 // ---------------------------------------------------------------------------
 // sat(a b + c) with one rounding
 __device__ __forceinline__ float fmasat(float a, float b, float c)
@@ -38,22 +38,12 @@ __device__ __forceinline__ float fmasat(float a, float b, float c)
     asm("fma.rn.ftz.sat.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
 }
-__device__ __forceinline__ double fmasat(double a, double b, double c)
-{
-    // the clamp to [0, 1] on the bits (the integer pipes, not the FP64
-    // one): a non-negative double orders like its bit pattern; u <= 0 and
-    // NaN give 0, as the f32 .sat form
-    const double u = ::fma(a, b, c);
-    const long long k = __double_as_longlong(u);
-    return k <= 0 ? 0.0 : (k >= 0x3ff0000000000000LL ? (k > 0x7ff0000000000000LL ? 0.0 : 1.0) : u);
-}
 __device__ __forceinline__ float max3(float a, float b, float c)
 {
     float r;
     asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
 }
-__device__ __forceinline__ double max3(double a, double b, double c) { return ::vmax(a, ::vmax(b, c)); }
 
 template <typename V>
 struct VOps;
@@ -96,20 +86,6 @@ struct VOps<float> {
     __device__ __forceinline__ static float zero() { return 0.f; }
 };
 
-template <>
-struct VOps<double> {
-    typedef double S;
-    static constexpr int W = 1;
-    __device__ __forceinline__ static double splat(double a) { return a; }
-    __device__ __forceinline__ static double fma(double a, double b, double c) { return ::fma(a, b, c); }
-    __device__ __forceinline__ static double mul(double a, double b) { return a * b; }
-    __device__ __forceinline__ static double add(double a, double b) { return a + b; }
-    __device__ __forceinline__ static double sub(double a, double b) { return a - b; }
-    __device__ __forceinline__ static double fsat(double a, double b, double c) { return fmasat(a, b, c); }
-    __device__ __forceinline__ static double vmin(double a, double b) { return ::vmin(a, b); }
-    __device__ __forceinline__ static double zero() { return 0.0; }
-};
-
 // per-line weights of the saturating form
 template <typename V>
 struct LineW {
@@ -124,14 +100,6 @@ template <int N>
 __device__ __forceinline__ float line_max(const float (&x)[N])
 {
     return fmaxf(tree_max<N>(x), 0.f);
-}
-template <int N>
-__device__ __forceinline__ double line_max(const double (&x)[N])
-{
-    double m = 0.0;
-#pragma unroll
-    for (int j = 0; j < N; ++j) m = ::vmax(m, x[j]);
-    return m;
 }
 // tree of 3-input maxima (short dependency chain)
 template <int N>
@@ -165,7 +133,6 @@ __device__ __forceinline__ float2 line_max(const float2 (&x)[N])
 }
 
 __device__ __forceinline__ float recip(float a) { return __frcp_rn(a); }
-__device__ __forceinline__ double recip(double a) { return __drcp_rn(a); }
 
 // weights from (c0, c1, c2), direction and the line maximum, one component
 template <typename S>
@@ -247,37 +214,6 @@ __device__ __forceinline__ V update_line(V (&x)[N], const LineW<V> &w, bool neg)
         }
         return PERIODIC ? z : phnext;
     }
-}
-
-// FP64 line update in the saturating form for any line maximum.  For a line
-// whose maximum lies below 2^-968 (subnormal or barely normal) the reciprocal
-// -1/F and the weights A1, A2 would overflow or lose their significant bits;
-// such a line is swept scaled by 2^968 and scaled back.  The PFC update is
-// positively homogeneous of degree one (scaling the line scales every face
-// flux), and a power of two scales without rounding, so the scaled sweep is
-// the same update; only the final scaling back rounds, into the subnormal
-// range, as the store of the unscaled result would.
-template <int N, bool PERIODIC>
-__device__ __forceinline__ double update_line_f64(double (&x)[N], double c0, double c1, double c2,
-                                                  int neg)
-{
-    constexpr double UP = 0x1p+968, DOWN = 0x1p-968;
-    double finf = line_max(x);
-    const bool tiny = finf > 0.0 && finf < DOWN;
-    if (tiny) {
-#pragma unroll
-        for (int j = 0; j < N; ++j) x[j] *= UP;
-        finf *= UP;
-    }
-    LineW<double> w;
-    weights1<double>(c0, c1, c2, neg, finf, w.K0, w.A1, w.A2, w.ninvF);
-    double lost = update_line<double, N, PERIODIC>(x, w, neg);
-    if (tiny) {
-#pragma unroll
-        for (int j = 0; j < N; ++j) x[j] *= DOWN;
-        lost *= DOWN;
-    }
-    return lost;
 }
 
 }  // namespace vpline

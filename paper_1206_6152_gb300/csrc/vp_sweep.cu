@@ -365,27 +365,26 @@ __global__ void k_coef_step(LineCoef<T> *__restrict__ kick, const double *__rest
 }
 
 // ---------------------------------------------------------------------------
-// rho(x) = dv^3 sum_v f (Sec. 2.2): one CTA per velocity cube, compensated
+// rho(x) = dv^3 sum_v f (Sec. 2.2), compensated: one CTA per velocity cube
 // ---------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(256) k_density(const T *__restrict__ f, long long np, int nvc,
+__global__ void __launch_bounds__(256) k_density(const float *__restrict__ f, long long np, int nvc,
                                                 double dvol, double *__restrict__ rho)
 {
-    __shared__ Acc<T> red[32];
+    __shared__ Acc<float> red[32];
     for (long long cell = blockIdx.x; cell < np; cell += gridDim.x) {
-        const T *q = f + cell * (long long)nvc;
-        Acc<T> a;
-        if (sizeof(T) == 4 && (nvc & 3) == 0) {
+        const float *q = f + cell * (long long)nvc;
+        Acc<float> a;
+        if ((nvc & 3) == 0) {
             // four independent compensated sums (one per float4 lane) for
             // memory-level parallelism, merged at the end
-            Acc<T> b, c2, d;
+            Acc<float> b, c2, d;
             const float4 *q4 = reinterpret_cast<const float4 *>(q);
             for (int e = threadIdx.x; e < nvc / 4; e += blockDim.x) {
                 const float4 v = q4[e];
-                a.add((T)v.x);
-                b.add((T)v.y);
-                c2.add((T)v.z);
-                d.add((T)v.w);
+                a.add(v.x);
+                b.add(v.y);
+                c2.add(v.z);
+                d.add(v.w);
             }
             a.merge(b);
             c2.merge(d);
@@ -396,6 +395,33 @@ __global__ void __launch_bounds__(256) k_density(const T *__restrict__ f, long l
         a = block_merge(a, red);
         if (threadIdx.x == 0) rho[cell] = a.value() * dvol;
         __syncthreads();
+    }
+}
+
+// FP64: WARP, one warp per cube, else one CTA.  Bound by the FP64 pipe (four
+// instructions per cell); merging 256 threads' sums costs a warp as much as 16
+// cells of its own, so cubes go to single warps where there are enough of them
+// to fill the SMs (16 warps each).
+template <bool WARP>
+__global__ void __launch_bounds__(256) k_density_f64(const double *__restrict__ f, long long np,
+                                                    int nvc, double dvol, double *__restrict__ rho)
+{
+    __shared__ Acc<double> red[32];
+    const int per = WARP ? 32 : blockDim.x, lane = threadIdx.x % per;
+    const long long groups = (long long)gridDim.x * (blockDim.x / per);
+    for (long long cell = (long long)blockIdx.x * (blockDim.x / per) + threadIdx.x / per; cell < np;
+         cell += groups) {
+        const double *q = f + cell * (long long)nvc;
+        Acc<double> a;
+#pragma unroll 4
+        for (int e = lane; e < nvc; e += per) a.add(q[e]);
+        if (WARP) {
+            for (int d = 16; d > 0; d >>= 1) a.shfl_merge(d);
+        } else {
+            a = block_merge(a, red);
+            __syncthreads();
+        }
+        if (lane == 0) rho[cell] = a.value() * dvol;
     }
 }
 
@@ -643,7 +669,7 @@ cudaError_t launch_kick(vp_ctx *c, void *f, const void *coef_a, const void *coef
 {
     if (vp_kick_fast_ok(c)) return launch_kick_fast(c, f, coef_a, coef_b, nsweeps, first_axis);
     if (vp_kick_big_ok(c)) return launch_kick_big(c, f, coef_a, coef_b, nsweeps, first_axis);
-    if (vp_kick_f64_ok(c)) return launch_kick_f64(c, f, coef_a, coef_b, nsweeps, first_axis, nullptr);
+    if (vp_kick_lines_ok(c)) return launch_kick_lines(c, f, coef_a, coef_b, nsweeps, first_axis, f);
     if (c->isdouble)
         return launch_kick_dispatch<double>(c, (double *)f, (const LineCoef<double> *)coef_a,
                                             (const LineCoef<double> *)coef_b, nsweeps,
@@ -659,8 +685,8 @@ cudaError_t launch_sweep_into(vp_ctx *c, const void *src, void *dst, int axis, c
         return launch_kick_fast(c, const_cast<void *>(src), coef, nullptr, 1, axis - 3, dst);
     if (axis >= 3 && vp_kick_big_ok(c))
         return launch_kick_big(c, const_cast<void *>(src), coef, nullptr, 1, axis - 3, dst);
-    if (axis >= 3 && vp_kick_f64_ok(c))
-        return launch_kick_f64(c, const_cast<void *>(src), coef, nullptr, 1, axis - 3, dst);
+    if (axis >= 3 && vp_kick_lines_ok(c))
+        return launch_kick_lines(c, src, coef, nullptr, 1, axis - 3, dst);
     if (axis < 3 && vp_drift_fast_ok(c, axis) && drift_alpha_bound < 1.0)
         return launch_drift_fast(c, const_cast<void *>(src), axis, coef, nullptr, dst);
     if (axis < 3 && vp_drift_lines_ok(c, axis) && drift_alpha_bound < 1.0)
@@ -674,14 +700,20 @@ cudaError_t launch_sweep_into(vp_ctx *c, const void *src, void *dst, int axis, c
 
 cudaError_t launch_density(vp_ctx *c, const void *f, double *rho)
 {
-    long long grid = (long long)sm_count() * 8;
-    if (grid > c->np) grid = c->np;
-    if (c->isdouble)
-        k_density<double><<<(unsigned)grid, 256, 0, c->stream>>>((const double *)f, c->np,
-                                                                 (int)c->nvc, c->dvol_v, rho);
-    else
-        k_density<float><<<(unsigned)grid, 256, 0, c->stream>>>((const float *)f, c->np,
-                                                                (int)c->nvc, c->dvol_v, rho);
+    const long long cap = (long long)sm_count() * 8;
+    long long grid = c->np < cap ? c->np : cap;
+    if (!c->isdouble) {
+        k_density<<<(unsigned)grid, 256, 0, c->stream>>>((const float *)f, c->np, (int)c->nvc, c->dvol_v,
+                                                         rho);
+    } else if (c->np >= 16LL * sm_count()) {
+        grid = (c->np + 7) / 8;
+        if (grid > cap) grid = cap;
+        k_density_f64<true><<<(unsigned)grid, 256, 0, c->stream>>>((const double *)f, c->np, (int)c->nvc,
+                                                                   c->dvol_v, rho);
+    } else {
+        k_density_f64<false><<<(unsigned)grid, 256, 0, c->stream>>>((const double *)f, c->np, (int)c->nvc,
+                                                                    c->dvol_v, rho);
+    }
     return cudaGetLastError();
 }
 

@@ -64,3 +64,29 @@ def test_drift_lines_match_oracle(n, space_bc, dtype):
         w = I.small_maxwell(n=tuple(shape), nv=nv, dtype=dtype, space_bc=space_bc)
         h, v = w.dx[axis], max(abs(w.vlo[axis]), abs(w.vhi[axis]))
         compare_sweep(w, axis, (0.7 * h / v, -0.97 * h / v, 2.3 * h / v), 10 * n + axis)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("n", [1, 2, 15, 16, 17, 32, 33, 64, 65])
+def test_kick_lines_match_oracle(n, dtype):
+    for axis in range(3):
+        nv = [5, 6, 7]
+        nv[axis] = n
+        w = I.small_maxwell(n=(3, 2, 5), nv=tuple(nv), dtype=dtype)
+        # accelerations of both signs: |shift| below a cell, and up to several
+        h = w.dv[axis]
+        compare_sweep(w, 3 + axis, (0.25 * h, -0.3 * h, 1.7 * h), 100 * n + axis)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,nv", [((16, 16, 10), (3, 2, 2)), ((2, 2, 3), (17, 16, 16))])
+def test_fp64_density_matches_oracle(n, nv):
+    """One warp per cube (many cubes) and one CTA per cube (few)."""
+    from paper_1206_6152_gb300.vlasov import VlasovPoisson, config_of
+    w = I.small_maxwell(n=n, nv=nv, dtype="f64")
+    f0 = np.random.default_rng(3).random(w.shape) ** 20        # widely spread values
+    with VlasovPoisson(config_of(w), torch.from_numpy(f0).to(DEV)) as sim:
+        rho = sim.density().cpu().numpy()
+    ref = O.density(f0, O.Grid.of(w))
+    assert np.abs(rho - ref).max() <= 4e-16 * ref.max()
