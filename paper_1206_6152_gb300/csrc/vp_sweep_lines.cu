@@ -20,6 +20,14 @@
 //    whole-cell shift takes the generic in-place routine.  FP64 cubes go
 //    through it one launch per sweep: at 16 bytes per cell the sweep is bound by
 //    the FP64 pipe alone.
+//  * k_kick_blocks: FP32 cubes in blocks of vx planes in shared memory: whole
+//    cubes, all sweeps of a kick in one pass, where they fit (220 KB); larger
+//    ones as one pass per vx sweep (k_kick_lines) and one per run of vy and vz
+//    sweeps (both inside a vx plane).  Bound by issue (about 22 instructions
+//    per cell and sweep: 15 of the flux and update, the rest loads, stores and
+//    the line's end).  Fused six-sweep kick: 24 x 28 x 26 cubes (554 MB of
+//    traffic) 1.83 -> 1.14 ms, 40^3 (1.0 GB) 5.1 -> 2.5 ms, 64^3 (537 MB) 2.56
+//    -> 1.15 ms against the shared-memory lines of vp_sweep.cu.
 #include <cuda_runtime.h>
 
 #include "vp_clamp_line.cuh"
@@ -33,30 +41,42 @@ int vp_sm_count();
 
 namespace {
 
-// What a thread's lines lose through the outflow ends, over all of its lines:
-// merging a CTA's threads takes about 50 FP64 instructions a warp, so it is
-// done once per CTA of a grid that just fills the SMs, not once per line.
+// What a thread's lines lose through the outflow ends, over all of its lines.
+// FP32 sums are kept and merged as double-floats on the FP32 pipe, one FP64
+// addition per warp at the end.  FP64: merging a CTA's threads takes about 50
+// FP64 instructions a warp, so it is done once per CTA of a grid that just
+// fills the SMs, not once per line.
 template <typename T>
 struct Lost;
 template <>
 struct Lost<float> {
     Acc<float> a;
     __device__ __forceinline__ void add(float v) { a.add(v); }
-    __device__ __forceinline__ double value() const { return a.value(); }
 };
 template <>
 struct Lost<double> {
     double a = 0.0;
     __device__ __forceinline__ void add(double v) { a += v; }
-    __device__ __forceinline__ double value() const { return a; }
 };
 
-template <typename T>
-__device__ __forceinline__ void add_lost(const Lost<T> &lost, double *lost_out)
+__device__ __forceinline__ void add_lost(Lost<float> lost, double *lost_out)
+{
+    __shared__ double red[32];
+    for (int d = 16; d > 0; d >>= 1) lost.a.shfl_merge(d);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = lost.a.value();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double s = 0.0;
+        for (int w = 0; w < (int)(blockDim.x + 31) / 32; ++w) s += red[w];
+        if (s != 0.0) atomicAdd(lost_out, s);
+    }
+}
+
+__device__ __forceinline__ void add_lost(const Lost<double> &lost, double *lost_out)
 {
     __shared__ Acc<double> red[32];
     Acc<double> a;
-    a.add(lost.value());
+    a.add(lost.a);
     a = block_merge(a, red);
     if (threadIdx.x == 0 && a.value() != 0.0) atomicAdd(lost_out, a.value());
 }
@@ -160,6 +180,131 @@ __global__ void __launch_bounds__(128) k_kick_lines(const T *src, T *dst,
     add_lost(lost, lost_out);
 }
 
+// one sweep of one FP32 line: n cells from p to w, element strides ps and ws
+// (both at the line's upwind end)
+template <int NMAX>
+__device__ __forceinline__ float sweep_line(const float *p, int ps, float *w, int ws, int n,
+                                            const LineCoef<float> &cf)
+{
+    float x[NMAX + 1];
+    x[0] = *p;
+#pragma unroll
+    for (int j = 1; j <= NMAX; ++j) {
+        p += ps;
+        x[j] = j < n ? *p : 0.f;
+    }
+    return clamp_line<float, NMAX, false>(x, n, 0.f, 0.f, cf.c0, cf.c1, cf.c2, [&](int, float v) {
+        *w = v;
+        w += ws;
+    });
+}
+
+// A block of G vx planes of a velocity cube (all of them: the whole cube) in
+// shared memory, rows at pitch nz | 1 (rows and columns free of bank
+// conflicts), one line per thread at a time.
+struct Block {
+    int g, ny, nz;         // planes, rows, cells per row
+    // the lines along axis va: how many, their length, line u's first cell and
+    // its step in an array of row pitch P
+    __device__ __forceinline__ int lines(int va) const { return va == 0 ? ny * nz : (va == 1 ? g * nz : g * ny); }
+    __device__ __forceinline__ int len(int va) const { return va == 0 ? g : (va == 1 ? ny : nz); }
+    __device__ __forceinline__ int step(int va, int P) const { return va == 0 ? ny * P : (va == 1 ? P : 1); }
+    __device__ __forceinline__ int first(int va, int u, int P) const
+    {
+        if (va == 2) return u * P;
+        const int r = u / nz, k = u - r * nz;
+        return (va == 0 ? r : r * ny) * P + k;
+    }
+};
+
+// f(e, tile offset) for every element e of rows of nz cells; element e lies in
+// row r at tile offset e + r (P - nz), r stepped along instead of divided out
+// (a division per element took longer than the sweeps: vz alone of 64^3
+// cubes, 537 MB of traffic, 1.06 -> 0.45 ms)
+template <class F>
+__device__ __forceinline__ void each_element(int count, int nz, F f)
+{
+    const int NT = blockDim.x, pad = (nz | 1) - nz, dr = NT / nz, dk = NT - dr * nz;
+    int r = threadIdx.x / nz, k = threadIdx.x - r * nz;
+#pragma unroll 4
+    for (int e = threadIdx.x; e < count; e += NT) {
+        f(e, e + r * pad);
+        r += dr;
+        k += dk;
+        if (k >= nz) { k -= nz; ++r; }
+    }
+}
+
+// nsweeps consecutive sweeps first_axis, first_axis + 1, ... (mod 3) of a
+// block, from src (global, pitch nz) into dst.  The first sweep reads vx or vy
+// lines, and the last one writes them, straight from and to global memory
+// (coalesced along vz); vz rows, and sweeps that move by whole cells, go
+// through the tile.  Starts and ends with the tile free.
+template <int NMAX>
+__device__ void sweep_block(const Block &B, const float *src, float *dst, float *tile,
+                            const LineCoef<float> *cf, int nsweeps, int first_axis, Lost<float> &lost)
+{
+    const int t = threadIdx.x, NT = blockDim.x, nz = B.nz, P = nz | 1, rows = B.g * B.ny;
+    auto whole = [&](int sw) { return (cf[sw].code >> 1) != 0; };
+    const bool in = first_axis < 2 && !whole(0);
+    if (!in) {
+        each_element(rows * nz, nz, [&](int e, int q) { tile[q] = src[e]; });
+        __syncthreads();
+    }
+    bool out = false;
+    for (int sw = 0; sw < nsweeps; ++sw) {
+        const int va = (first_axis + sw) % 3, n = B.len(va), L = B.lines(va), st = B.step(va, P);
+        const LineCoef<float> c = cf[sw];
+        const int neg = c.code & 1, sg = B.step(va, nz);
+        out = sw == nsweeps - 1 && va < 2 && !whole(sw);
+        if (whole(sw)) {
+            for (int u = t; u < L; u += NT) lost.add(kick_line_shifted(tile + B.first(va, u, P), st, n, c));
+        } else {
+            for (int u = t; u < L; u += NT) {
+                const int a = B.first(va, u, P) + (neg ? (n - 1) * st : 0);
+                const int b = va < 2 ? B.first(va, u, nz) + (neg ? (n - 1) * sg : 0) : 0;
+                const float *p = sw == 0 && in ? src + b : tile + a;
+                float *w = out ? dst + b : tile + a;
+                const int ps = sw == 0 && in ? sg : st, ws = out ? sg : st;
+                lost.add(sweep_line<NMAX>(p, neg ? -ps : ps, w, neg ? -ws : ws, n, c));
+            }
+        }
+        __syncthreads();
+    }
+    if (!out) {
+        each_element(rows * nz, nz, [&](int e, int q) { dst[e] = tile[q]; });
+        __syncthreads();
+    }
+}
+
+// FP32 cubes in blocks of G vx planes (G = nx: whole cubes), nsweeps <= 6
+// sweeps per block; tables ca for the first three sweeps of the kick, cb after
+// (k0: how many sweeps of the kick came before)
+template <int NMAX>
+__global__ void __launch_bounds__(512) k_kick_blocks(const float *src, float *dst,
+                                                    const LineCoef<float> *__restrict__ ca,
+                                                    const LineCoef<float> *__restrict__ cb, int k0,
+                                                    int nsweeps, int first_axis, int nx, int ny, int nz,
+                                                    int G, long long np, double *lost_out)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ LineCoef<float> scf[6];
+    const int per = (nx + G - 1) / G;
+    Lost<float> lost;
+    for (long long u = blockIdx.x; u < np * per; u += gridDim.x) {
+        const long long cell = u / per;
+        const int i0 = (int)(u - cell * per) * G;
+        if (threadIdx.x < nsweeps)
+            scf[threadIdx.x] = (k0 + (int)threadIdx.x < 3 ? ca : cb)[cell * 3 + (first_axis + threadIdx.x) % 3];
+        __syncthreads();
+        const Block B{nx - i0 < G ? nx - i0 : G, ny, nz};
+        const long long off = (cell * nx + i0) * ny * (long long)nz;
+        sweep_block<NMAX>(B, src + off, dst + off, reinterpret_cast<float *>(smem_raw), scf, nsweeps,
+                          first_axis, lost);
+    }
+    add_lost(lost, lost_out);
+}
+
 // CTAs of 128 threads, one line per thread at a time: as many as there are
 // lines for, or with persistent only those that fit on the GPU at once.  The
 // persistent grid pays where every CTA ends with a merge of its losses (FP64
@@ -192,6 +337,61 @@ cudaError_t kick_lines_t(vp_ctx *c, const T *src, T *dst, const LineCoef<T> *coe
     kern<<<grid, 128, 0, c->stream>>>(src, dst, coef, va, c->nv[0], c->nv[1], c->nv[2], c->np,
                                       &c->sc->lost);
     return cudaGetLastError();
+}
+
+cudaError_t kick_blocks(vp_ctx *c, const float *src, float *dst, const LineCoef<float> *ca,
+                        const LineCoef<float> *cb, int k0, int nsweeps, int first_axis, int G)
+{
+    const int nx = c->nv[0], ny = c->nv[1], nz = c->nv[2];
+    const size_t smem = (size_t)G * ny * (nz | 1) * sizeof(float);
+    int lmax = G * (ny > nz ? ny : nz);              // most lines of one sweep
+    if (G == nx && ny * nz > lmax) lmax = ny * nz;
+    // a CTA alone on its SM gets 16 warps, CTAs that share one 8 at most
+    int threads = (lmax + 31) / 32 * 32;
+    const int cap = smem > 110 * 1024 ? 512 : 256;
+    if (threads > cap) threads = cap;
+    auto kern = c->maxnv <= 16 ? k_kick_blocks<16> : (c->maxnv <= 32 ? k_kick_blocks<32> : k_kick_blocks<64>);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+    if (e != cudaSuccess) return e;
+    int per_sm = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) return cudaErrorInvalidConfiguration;
+    long long grid = (long long)per_sm * vp_sm_count();
+    const long long units = c->np * ((nx + G - 1) / G);
+    if (grid > units) grid = units;
+    kern<<<(unsigned)grid, threads, smem, c->stream>>>(src, dst, ca, cb, k0, nsweeps, first_axis, nx, ny,
+                                                       nz, G, c->np, &c->sc->lost);
+    return cudaGetLastError();
+}
+
+// FP32: whole cubes in one pass where they fit in shared memory; else one
+// pass per vx sweep (register lines) and one per run of vy and vz sweeps (both
+// inside a vx plane; blocks of enough planes for four warps of lines)
+cudaError_t kick_lines_f32(vp_ctx *c, const float *src, float *dst, const LineCoef<float> *ca,
+                           const LineCoef<float> *cb, int nsweeps, int first_axis)
+{
+    const int nx = c->nv[0], ny = c->nv[1], nz = c->nv[2];
+    if ((size_t)nx * ny * (nz | 1) * sizeof(float) <= 220 * 1024)
+        return kick_blocks(c, src, dst, ca, cb, 0, nsweeps, first_axis, nx);
+    int G = 128 / (ny < nz ? ny : nz);
+    if (G < 1) G = 1;
+    if (G > nx) G = nx;
+    for (int sw = 0; sw < nsweeps;) {
+        const int va = (first_axis + sw) % 3;
+        int run = 1;
+        cudaError_t e;
+        if (va == 0) {
+            e = kick_lines_t<float>(c, src, dst, sw < 3 ? ca : cb, 0);
+        } else {
+            if (va == 1 && sw + 1 < nsweeps) run = 2;
+            e = kick_blocks(c, src, dst, ca, cb, sw, run, va, G);
+        }
+        if (e != cudaSuccess) return e;
+        src = dst;              // the first pass reads src, the rest dst
+        sw += run;
+    }
+    return cudaSuccess;
 }
 
 template <typename T, bool PERIODIC>
@@ -243,15 +443,15 @@ cudaError_t launch_drift_lines(vp_ctx *c, const void *f, int axis, const void *c
     return drift_lines_t<float>(c, (const float *)f, axis, (const LineCoef<float> *)coef, (float *)fo);
 }
 
-// FP64 cubes with no axis longer than 64, one launch per sweep
-int vp_kick_lines_ok(const vp_ctx *c)
-{
-    return c->isdouble && c->maxnv <= 64;
-}
+// velocity cubes with no axis longer than 64
+int vp_kick_lines_ok(const vp_ctx *c) { return c->maxnv <= 64; }
 
 cudaError_t launch_kick_lines(vp_ctx *c, const void *f, const void *ca, const void *cb, int nsweeps,
                               int first_axis, void *fo)
 {
+    if (!c->isdouble)
+        return kick_lines_f32(c, (const float *)f, (float *)fo, (const LineCoef<float> *)ca,
+                              (const LineCoef<float> *)cb, nsweeps, first_axis);
     const double *src = (const double *)f;
     double *dst = (double *)fo;
     for (int sw = 0; sw < nsweeps; ++sw) {
