@@ -332,20 +332,6 @@ __global__ void __launch_bounds__(256) k_functional_grad(T *__restrict__ lam_f,
     }
 }
 
-// sum (rho - target)^2 (compensated), one CTA
-__global__ void k_misfit(const double *__restrict__ rho, const double *__restrict__ target,
-                         long long np, double *out)
-{
-    __shared__ Acc<double> red[32];
-    Acc<double> a;
-    for (long long t = threadIdx.x; t < np; t += blockDim.x) {
-        const double r = rho[t] - target[t];
-        a.add(r * r);
-    }
-    a = block_merge(a, red);
-    if (threadIdx.x == 0) out[0] = a.value();
-}
-
 // ---------------------------------------------------------------------------
 // register-line adjoint (line lengths 16/32/48/64, zero whole-cell shift):
 // the line of f, the output cotangent and the input cotangent live in
@@ -807,13 +793,8 @@ int vp_functional(vp_ctx *c, int kind, const double *target, void *lambda_f, dou
     const int T = 256;
     VP_CUDA_TRY(launch_density(c, c->f, c->rho2));
     double *sums = c->red + 2 * c->np;
-    if (kind == 0) {
-        VP_CUDA_TRY(launch_field_solve(c, c->rho2, nullptr));
-        VP_CUDA_TRY(launch_dot_rho_phi(c, c->rho2, sums));
-    } else {
-        k_misfit<<<1, 1024, 0, c->stream>>>(c->rho2, target, c->np, sums);
-        VP_CUDA_TRY(cudaGetLastError());
-    }
+    if (kind == 0) VP_CUDA_TRY(launch_field_solve(c, c->rho2, nullptr));
+    VP_CUDA_TRY(launch_energy_sums(c, nullptr, c->rho2, kind == 1 ? target : nullptr, sums));
     const double scale = c->dvol_v * c->dvol_x;
     long long grid = 8LL * vp_sm_count();
     if (grid > c->np) grid = c->np;
@@ -827,7 +808,7 @@ int vp_functional(vp_ctx *c, int kind, const double *target, void *lambda_f, dou
             c->fn[2], scale, c->np);
     VP_CUDA_TRY(cudaGetLastError());
     double h;
-    VP_CUDA_TRY(cudaMemcpyAsync(&h, sums, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+    VP_CUDA_TRY(cudaMemcpyAsync(&h, sums + 2, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     VP_CUDA_TRY(cudaStreamSynchronize(c->stream));
     if (J_out) *J_out = 0.5 * h * c->dvol_x;
     return VP_OK;

@@ -433,7 +433,7 @@ int init_ctx(const vp_config *cfg, void *f_dev, void *cuda_stream, vp_ctx **out)
         (r = dalloc(&c->coef_kick1, cs * 3 * c->np)) ||
         (r = dalloc(&c->coef_kick2, cs * 3 * c->np)) ||
         (r = dalloc(&c->coef_drift, cs * 3 * c->maxnv)) ||
-        (r = dalloc((void **)&c->red, sizeof(double) * (2 * c->np + 64))) ||
+        (r = dalloc((void **)&c->red, sizeof(double) * vp_energy_scratch(c->np))) ||
         (r = dalloc((void **)&c->sc, sizeof(DevScalars))))
         return fail(r);
     if (vp_rho_fuse_ok(c)) {
@@ -567,14 +567,12 @@ int vp_energy(vp_ctx *c, double out[5])
 {
     if (!c || !out) return VP_ERR_ARG;
     if (!c->f) return VP_ERR_STATE;
-    // M and K: per-cell partials, then a compensated reduction
-    VP_CUDA_TRY(launch_energy_partials(c, c->f, c->red));
-    double *sums = c->red + 2 * c->np;
-    VP_CUDA_TRY(launch_reduce_strided(c, c->red, c->np, 2, sums));
-    // U: the potential of the current f
-    VP_CUDA_TRY(launch_density(c, c->f, c->rho2));
+    // one read of f: per-cell partials of M and K and the density, whose
+    // potential gives U; then compensated sums over the cells
+    VP_CUDA_TRY(launch_energy_partials(c, c->f, c->red, c->rho2));
     VP_CUDA_TRY(launch_field_solve(c, c->rho2, nullptr));
-    VP_CUDA_TRY(launch_dot_rho_phi(c, c->rho2, sums + 2));
+    double *sums = c->red + 2 * c->np;
+    VP_CUDA_TRY(launch_energy_sums(c, c->red, c->rho2, nullptr, sums));
     double h[3];
     VP_CUDA_TRY(cudaMemcpyAsync(h, sums, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
     VP_CUDA_TRY(cudaMemcpyAsync(c->sc_host, c->sc, sizeof(DevScalars), cudaMemcpyDeviceToHost,

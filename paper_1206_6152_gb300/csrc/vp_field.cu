@@ -372,34 +372,6 @@ __global__ void k_copy_box(const double *__restrict__ src, double *__restrict__ 
     dst[t] = src[((long long)i * f1 + j) * f2 + k];
 }
 
-// out[0] += sum rho * phi_box (compensated), one CTA
-__global__ void k_dot_rho_phi(const double *__restrict__ rho, const double *__restrict__ phi,
-                              int n0, int n1, int n2, int f1, int f2, double *out)
-{
-    __shared__ Acc<double> red[32];
-    const long long np = (long long)n0 * n1 * n2;
-    Acc<double> a;
-    for (long long t = threadIdx.x; t < np; t += blockDim.x) {
-        const int k = (int)(t % n2);
-        const int j = (int)((t / n2) % n1);
-        const int i = (int)(t / ((long long)n1 * n2));
-        a.add(rho[t] * phi[((long long)i * f1 + j) * f2 + k]);
-    }
-    a = block_merge(a, red);
-    if (threadIdx.x == 0) out[0] = a.value();
-}
-
-// out[j] = sum_i in[i * stride + j] for j < stride (compensated), one CTA per j
-__global__ void k_reduce_strided(const double *__restrict__ in, long long n, int stride,
-                                 double *__restrict__ out)
-{
-    __shared__ Acc<double> red[32];
-    Acc<double> a;
-    for (long long i = threadIdx.x; i < n; i += blockDim.x) a.add(in[i * stride + blockIdx.x]);
-    a = block_merge(a, red);
-    if (threadIdx.x == 0) out[blockIdx.x] = a.value();
-}
-
 inline unsigned blocks_for(long long n, int threads) { return (unsigned)((n + threads - 1) / threads); }
 
 FFTPlan plan_of(const FFTAxis &A)
@@ -585,20 +557,5 @@ cudaError_t launch_copy_phi_box(vp_ctx *c, double *dst)
 {
     k_copy_box<<<blocks_for(c->np, 256), 256, 0, c->stream>>>(c->phi, dst, c->n[0], c->n[1],
                                                               c->n[2], c->fn[1], c->fn[2]);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_dot_rho_phi(vp_ctx *c, const double *rho, double *out)
-{
-    k_dot_rho_phi<<<1, 1024, 0, c->stream>>>(rho, c->phi, c->n[0], c->n[1], c->n[2], c->fn[1],
-                                             c->fn[2], out);
-    return cudaGetLastError();
-}
-
-// sums of `stride` interleaved sequences of length n
-cudaError_t launch_reduce_strided(vp_ctx *c, const double *in, long long n, int stride,
-                                  double *out)
-{
-    k_reduce_strided<<<stride, 1024, 0, c->stream>>>(in, n, stride, out);
     return cudaGetLastError();
 }

@@ -84,7 +84,7 @@ struct vp_ctx {
     void *coef_drift;           // LineCoef<T>[3][maxnv]
     int maxnv;
     double *vc[3];              // velocity cell centres (device)
-    double *red;                // reduction scratch (2 np + 64 doubles)
+    double *red;                // reduction scratch (vp_energy_scratch doubles)
     double *rho2;               // density of the current f for diagnostics
     double *rho_part;           // density partials of the fused x drift
     int rho_nparts;
@@ -140,11 +140,14 @@ cudaError_t launch_field_solve(vp_ctx *c, const double *rho, double *g_out);
 cudaError_t launch_field_step(vp_ctx *c, const double *rho, void *kick, int next);
 // out = G * in on the FFT grid (real); whole: in covers it, else the box
 cudaError_t launch_convolve(vp_ctx *c, const double *in, int whole, double *out);
-cudaError_t launch_energy_partials(vp_ctx *c, const void *f, double *partials);
+// per spatial cell sum f, sum f |v|^2 (interleaved) and the density
+cudaError_t launch_energy_partials(vp_ctx *c, const void *f, double *partials, double *rho);
+// out[0], out[1]: sums of partials (may be null); out[2]: sum rho phi, or with
+// target sum (rho - target)^2
+cudaError_t launch_energy_sums(vp_ctx *c, const double *partials, const double *rho,
+                               const double *target, double *out);
+size_t vp_energy_scratch(long long np);     // doubles of c->red
 cudaError_t launch_copy_phi_box(vp_ctx *c, double *dst);
-cudaError_t launch_dot_rho_phi(vp_ctx *c, const double *rho, double *out2);
-cudaError_t launch_reduce_strided(vp_ctx *c, const double *in, long long n, int stride,
-                                  double *out);
 int vp_sm_count();
 
 // register-line kernels (vp_sweep_fast.cu)

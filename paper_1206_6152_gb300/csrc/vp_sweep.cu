@@ -425,36 +425,6 @@ __global__ void __launch_bounds__(256) k_density_f64(const double *__restrict__ 
     }
 }
 
-// per spatial cell: sum f and sum f |v|^2 (FP64, Neumaier) -> partials[2*cell]
-template <typename T>
-__global__ void __launch_bounds__(256) k_energy_partials(const T *__restrict__ f, long long np,
-                                                        int nvx, int nvy, int nvz,
-                                                        const double *vcx, const double *vcy,
-                                                        const double *vcz, double *partials)
-{
-    __shared__ Acc<double> red[32];
-    const int nvc = nvx * nvy * nvz;
-    for (long long cell = blockIdx.x; cell < np; cell += gridDim.x) {
-        const T *q = f + cell * (long long)nvc;
-        Acc<double> a0, a2;
-        for (int e = threadIdx.x; e < nvc; e += blockDim.x) {
-            const int i = e / (nvy * nvz);
-            const int r = e - i * nvy * nvz;
-            const int j = r / nvz, k = r - j * nvz;
-            const double v2 = vcx[i] * vcx[i] + vcy[j] * vcy[j] + vcz[k] * vcz[k];
-            const double x = (double)q[e];
-            a0.add(x);
-            a2.add(x * v2);
-        }
-        a0 = block_merge(a0, red);
-        if (threadIdx.x == 0) partials[2 * cell] = a0.value();
-        __syncthreads();
-        a2 = block_merge(a2, red);
-        if (threadIdx.x == 0) partials[2 * cell + 1] = a2.value();
-        __syncthreads();
-    }
-}
-
 int sm_count()
 {
     static int n = 0;
@@ -714,20 +684,5 @@ cudaError_t launch_density(vp_ctx *c, const void *f, double *rho)
         k_density_f64<false><<<(unsigned)grid, 256, 0, c->stream>>>((const double *)f, c->np, (int)c->nvc,
                                                                     c->dvol_v, rho);
     }
-    return cudaGetLastError();
-}
-
-cudaError_t launch_energy_partials(vp_ctx *c, const void *f, double *partials)
-{
-    long long grid = (long long)sm_count() * 8;
-    if (grid > c->np) grid = c->np;
-    if (c->isdouble)
-        k_energy_partials<double><<<(unsigned)grid, 256, 0, c->stream>>>(
-            (const double *)f, c->np, c->nv[0], c->nv[1], c->nv[2], c->vc[0], c->vc[1],
-            c->vc[2], partials);
-    else
-        k_energy_partials<float><<<(unsigned)grid, 256, 0, c->stream>>>(
-            (const float *)f, c->np, c->nv[0], c->nv[1], c->nv[2], c->vc[0], c->vc[1], c->vc[2],
-            partials);
     return cudaGetLastError();
 }
