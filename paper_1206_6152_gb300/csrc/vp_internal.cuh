@@ -183,6 +183,13 @@ cudaError_t launch_drift_lines(vp_ctx *c, const void *f, int axis, const void *c
 int vp_kick_lines_ok(const vp_ctx *c);
 cudaError_t launch_kick_lines(vp_ctx *c, const void *f, const void *ca, const void *cb, int nsweeps,
                               int first_axis, void *fo);
+// the same for FP64 grids with few lines, one thread per cell, any shift
+// (vp_sweep_cells.cu)
+int vp_drift_cells_ok(const vp_ctx *c, int axis);
+cudaError_t launch_drift_cells(vp_ctx *c, const void *f, int axis, const void *coef, void *fo);
+int vp_kick_cells_ok(const vp_ctx *c);
+cudaError_t launch_kick_cells(vp_ctx *c, const void *f, const void *ca, const void *cb, int nsweeps,
+                              int first_axis, void *fo);
 // one sweep from src into dst (dst != src), used by the adjoint's replay;
 // kick tables [np][3], drift tables [3][maxnv]
 cudaError_t launch_sweep_into(vp_ctx *c, const void *src, void *dst, int axis, const void *coef,

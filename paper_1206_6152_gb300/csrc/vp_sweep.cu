@@ -627,7 +627,10 @@ cudaError_t launch_drift(vp_ctx *c, void *f, int axis, const void *coef, double 
 {
     const bool fast = vp_drift_fast_ok(c, axis) && max_alpha < 1.0;
     if (rho_part && !(fast && axis == 0 && vp_rho_fuse_ok(c))) return cudaErrorNotSupported;
+    // a periodic line of one cell: what leaves it comes back
+    if (c->n[axis] == 1 && c->periodic_space && !rho_part) return cudaSuccess;
     if (fast) return launch_drift_fast(c, f, axis, coef, rho_part);
+    if (vp_drift_cells_ok(c, axis)) return launch_drift_cells(c, f, axis, coef, f);
     if (vp_drift_lines_ok(c, axis) && max_alpha < 1.0) return launch_drift_lines(c, f, axis, coef, f);
     if (c->isdouble)
         return launch_drift_t<double>(c, (double *)f, axis, (const LineCoef<double> *)coef);
@@ -639,6 +642,7 @@ cudaError_t launch_kick(vp_ctx *c, void *f, const void *coef_a, const void *coef
 {
     if (vp_kick_fast_ok(c)) return launch_kick_fast(c, f, coef_a, coef_b, nsweeps, first_axis);
     if (vp_kick_big_ok(c)) return launch_kick_big(c, f, coef_a, coef_b, nsweeps, first_axis);
+    if (vp_kick_cells_ok(c)) return launch_kick_cells(c, f, coef_a, coef_b, nsweeps, first_axis, f);
     if (vp_kick_lines_ok(c)) return launch_kick_lines(c, f, coef_a, coef_b, nsweeps, first_axis, f);
     if (c->isdouble)
         return launch_kick_dispatch<double>(c, (double *)f, (const LineCoef<double> *)coef_a,
@@ -655,10 +659,13 @@ cudaError_t launch_sweep_into(vp_ctx *c, const void *src, void *dst, int axis, c
         return launch_kick_fast(c, const_cast<void *>(src), coef, nullptr, 1, axis - 3, dst);
     if (axis >= 3 && vp_kick_big_ok(c))
         return launch_kick_big(c, const_cast<void *>(src), coef, nullptr, 1, axis - 3, dst);
+    if (axis >= 3 && vp_kick_cells_ok(c))
+        return launch_kick_cells(c, src, coef, nullptr, 1, axis - 3, dst);
     if (axis >= 3 && vp_kick_lines_ok(c))
         return launch_kick_lines(c, src, coef, nullptr, 1, axis - 3, dst);
     if (axis < 3 && vp_drift_fast_ok(c, axis) && drift_alpha_bound < 1.0)
         return launch_drift_fast(c, const_cast<void *>(src), axis, coef, nullptr, dst);
+    if (axis < 3 && vp_drift_cells_ok(c, axis)) return launch_drift_cells(c, src, axis, coef, dst);
     if (axis < 3 && vp_drift_lines_ok(c, axis) && drift_alpha_bound < 1.0)
         return launch_drift_lines(c, src, axis, coef, dst);
     cudaError_t e = cudaMemcpyAsync(dst, src, (size_t)c->ncells * c->esize,
@@ -675,10 +682,12 @@ cudaError_t launch_density(vp_ctx *c, const void *f, double *rho)
     if (!c->isdouble) {
         k_density<<<(unsigned)grid, 256, 0, c->stream>>>((const float *)f, c->np, (int)c->nvc, c->dvol_v,
                                                          rho);
-    } else if (c->np >= 16LL * sm_count()) {
-        grid = (c->np + 7) / 8;
+    } else if (c->np >= 16LL * sm_count() || c->nvc <= 512) {
+        // (few small cubes: one warp per CTA, so that the warps spread over the SMs)
+        const int per = c->np >= 16LL * sm_count() ? 8 : 1;
+        grid = (c->np + per - 1) / per;
         if (grid > cap) grid = cap;
-        k_density_f64<true><<<(unsigned)grid, 256, 0, c->stream>>>((const double *)f, c->np, (int)c->nvc,
+        k_density_f64<true><<<(unsigned)grid, 32 * per, 0, c->stream>>>((const double *)f, c->np, (int)c->nvc,
                                                                    c->dvol_v, rho);
     } else {
         k_density_f64<false><<<(unsigned)grid, 256, 0, c->stream>>>((const double *)f, c->np, (int)c->nvc,

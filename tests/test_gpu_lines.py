@@ -120,3 +120,20 @@ def test_fp32_steps_of_any_cube_match_oracle(nv, whole_cell):
     # 18 sweeps, one FP32 rounding of about 6e-8 each
     assert np.abs(got - ref.f).sum() <= 4e-6 * np.abs(ref.f).sum()
     assert got.min() >= 0.0
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("space_bc", ["periodic", "outflow"])
+@pytest.mark.parametrize("n", [15, 18, 33, 64])
+def test_fp64_many_lines_match_oracle(n, space_bc):
+    """Lines enough to fill the GPU (21120 and more): one thread per line; the
+    tests above have few lines in FP64, which take one thread per cell."""
+    w = I.small_maxwell(n=(n, 4, 4), nv=(12, 11, 10), dtype="f64", space_bc=space_bc)
+    h, v = w.dx[0], max(abs(w.vlo[0]), abs(w.vhi[0]))
+    compare_sweep(w, 0, (0.7 * h / v, -0.97 * h / v), n)
+    if space_bc == "outflow":
+        return
+    w = I.small_maxwell(n=(16, 8, 8), nv=(5, 6, n), dtype="f64")
+    compare_sweep(w, 5, (0.25 * w.dv[2], -1.1 * w.dv[2]), n + 1)
+    w = I.small_maxwell(n=(16, 8, 8), nv=(n, 5, 6), dtype="f64")
+    compare_sweep(w, 3, (0.25 * w.dv[0], -1.1 * w.dv[0]), n + 2)
