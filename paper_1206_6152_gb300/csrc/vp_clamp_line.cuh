@@ -52,15 +52,53 @@ __device__ __forceinline__ T clamp_flux(T dm, T f0, T dp, T finf, T c0, T c1, T 
     return vmin(vmax(phi, T(0)), f0);
 }
 
+// Loops over the cells go in groups of GR, unrolled: whole groups without any
+// test per cell, then one partial group.  GR = 1 (a branch out after the last
+// cell) is what FP64 needs, as instructions of cells past the end would take FP64
+// pipe slots even where predicated off, and what serves FP32 lines best that are
+// bound by HBM or much shorter than NMAX; GR = 4 serves the issue-bound kicks.
+
+// cells 0 .. n - 1 of a line by get() in turn, and what lies behind them (the
+// first cell, or 0)
+template <typename T, int NMAX, bool PERIODIC, int GR, class G>
+__device__ __forceinline__ void load_line(T (&x)[NMAX + 1], int n, G get)
+{
+    if constexpr (GR == 1) {
+        x[0] = get();
+#pragma unroll
+        for (int j = 1; j <= NMAX; ++j) x[j] = j < n ? get() : (PERIODIC ? x[0] : T(0));
+    } else {
+#pragma unroll
+        for (int j = 0; j < NMAX; j += GR) {
+            if (j + GR <= n) {
+#pragma unroll
+                for (int i = 0; i < GR; ++i) x[j + i] = get();
+            } else {
+                // (every x is set on every path: registers left undefined
+                // past the end would be held over from the line before)
+#pragma unroll
+                for (int i = 0; i < GR; ++i) {
+                    x[j + i] = PERIODIC && j + i ? x[0] : T(0);
+                    if (j + i < n) x[j + i] = get();
+                }
+            }
+        }
+        x[NMAX] = PERIODIC ? x[0] : T(0);
+    }
+}
+
 // maximum of the line and 0
-template <typename T, int NMAX>
+template <typename T, int NMAX, int GR>
 __device__ __forceinline__ T clamp_line_max(const T (&x)[NMAX + 1], int n)
 {
     T m = T(0);
 #pragma unroll
-    for (int j = 0; j < NMAX; ++j) {
-        if (j >= n) break;
-        m = vmax(m, x[j]);
+    for (int j = 0; j < NMAX; j += GR) {
+        if (GR == 1 && j >= n) break;
+        if (j < n) {                    // (a partial group's pads are 0 or x[0])
+#pragma unroll
+            for (int i = 0; i < GR; ++i) m = vmax(m, x[j + i]);
+        }
     }
     return m;
 }
@@ -69,24 +107,36 @@ __device__ __forceinline__ T clamp_line_max(const T (&x)[NMAX + 1], int n)
 // increasing j, after every cell of the line has been read.  PERIODIC: fm1,
 // fm2 are the line's last and last but one cells.  Returns the last cell's
 // flux (what leaves an outflow line).
-template <typename T, int NMAX, bool PERIODIC, class P>
+template <typename T, int NMAX, bool PERIODIC, int GR, class P>
 __device__ __forceinline__ T clamp_line(const T (&x)[NMAX + 1], int n, T fm1, T fm2, T c0, T c1, T c2,
                                         P put)
 {
-    const T finf = clamp_line_max<T, NMAX>(x, n);
+    const T finf = clamp_line_max<T, NMAX, GR>(x, n);
     T dm = x[0], phm = T(0);                    // outflow: f_{-1} = 0
     if (PERIODIC) {
         dm = x[0] - fm1;
         phm = clamp_flux(fm1 - fm2, fm1, dm, finf, c0, c1, c2);
     }
-#pragma unroll
-    for (int j = 0; j < NMAX; ++j) {
-        if (j >= n) break;          // a branch: cells past the end take no issue slots
-        const T dp = x[j + 1] - x[j];
-        const T ph = clamp_flux(dm, x[j], dp, finf, c0, c1, c2);
-        put(j, (x[j] - ph) + phm);
+    auto cell = [&](int i) {
+        const T dp = x[i + 1] - x[i];
+        const T ph = clamp_flux(dm, x[i], dp, finf, c0, c1, c2);
+        put(i, (x[i] - ph) + phm);
         phm = ph;
         dm = dp;
+    };
+#pragma unroll
+    for (int j = 0; j < NMAX; j += GR) {
+        if constexpr (GR == 1) {
+            if (j >= n) break;
+            cell(j);
+        } else if (j + GR <= n) {
+#pragma unroll
+            for (int i = 0; i < GR; ++i) cell(j + i);
+        } else if (j < n) {
+#pragma unroll
+            for (int i = 0; i < GR; ++i)
+                if (j + i < n) cell(j + i);
+        }
     }
     return phm;
 }

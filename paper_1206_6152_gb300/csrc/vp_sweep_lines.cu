@@ -23,11 +23,13 @@
 //  * k_kick_blocks: FP32 cubes in blocks of vx planes in shared memory: whole
 //    cubes, all sweeps of a kick in one pass, where they fit (220 KB); larger
 //    ones as one pass per vx sweep (k_kick_lines) and one per run of vy and vz
-//    sweeps (both inside a vx plane).  Bound by issue (about 22 instructions
-//    per cell and sweep: 15 of the flux and update, the rest loads, stores and
-//    the line's end).  Fused six-sweep kick: 24 x 28 x 26 cubes (554 MB of
-//    traffic) 1.83 -> 1.14 ms, 40^3 (1.0 GB) 5.1 -> 2.5 ms, 64^3 (537 MB) 2.56
-//    -> 1.15 ms against the shared-memory lines of vp_sweep.cu.
+//    sweeps (both inside a vx plane).  Bound by issue (about 30 instructions per
+//    cell and sweep, 15 of them the flux and update), so the line loops go in
+//    whole groups of four cells where NMAX fits the lines, and the tile is
+//    addressed as shared memory.  Fused six-sweep kick against the shared-memory
+//    lines of vp_sweep.cu: 24 x 28 x 26 cubes (554 MB of traffic) 1.83 -> 0.93
+//    ms, 24^3 (764 MB) 2.78 -> 1.19 ms, 40^3 (1.0 GB) 5.1 -> 2.4 ms, 64^3 (537
+//    MB) 2.56 -> 1.18 ms.
 #include <cuda_runtime.h>
 
 #include "vp_clamp_line.cuh"
@@ -81,6 +83,17 @@ __device__ __forceinline__ void add_lost(const Lost<double> &lost, double *lost_
     if (threadIdx.x == 0 && a.value() != 0.0) atomicAdd(lost_out, a.value());
 }
 
+// *p, and p stepped on through an opaque register (the compiler would
+// otherwise keep every address of a line live from its loads to its stores)
+template <typename T, typename S>
+__device__ __forceinline__ T next(const T *&p, S st)
+{
+    const T v = *p;
+    p += st;
+    asm volatile("" : "+l"(p));
+    return v;
+}
+
 struct LinesGeom {
     int n;                     // cells per line
     long long cell_stride;     // spatial-cell stride along the line
@@ -113,21 +126,17 @@ __global__ void __launch_bounds__(128) k_drift_lines(const T *f, const LineCoef<
         const long long st = neg ? -step : step;
         T x[NMAX + 1];
         const T *p = f + off;
-        x[0] = *p;
-#pragma unroll
-        for (int j = 1; j <= NMAX; ++j) {
-            p += st;
-            x[j] = j < n ? *p : (PERIODIC ? x[0] : T(0));
-        }
+        load_line<T, NMAX, PERIODIC, 1>(x, n, [&]() { return next(p, st); });
         T fm1 = T(0), fm2 = T(0);
         if (PERIODIC) {
             fm1 = f[off + (n - 1) * st];
             fm2 = f[off + (n > 1 ? n - 2 : 0) * st];
         }
         T *w = fo + off;
-        const T out = clamp_line<T, NMAX, PERIODIC>(x, n, fm1, fm2, cf.c0, cf.c1, cf.c2, [&](int, T u) {
+        const T out = clamp_line<T, NMAX, PERIODIC, 1>(x, n, fm1, fm2, cf.c0, cf.c1, cf.c2, [&](int, T u) {
             *w = u;
             w += st;
+            asm volatile("" : "+l"(w));
         });
         if (!PERIODIC) lost.add(out);
         if (!drift_persistent<T, PERIODIC>()) break;
@@ -166,37 +175,14 @@ __global__ void __launch_bounds__(128) k_kick_lines(const T *src, T *dst,
         const T *p = src + off + (neg ? (n - 1) * step : 0);
         T *w = dst + off + (neg ? (n - 1) * step : 0);
         T x[NMAX + 1];
-        x[0] = *p;
-#pragma unroll
-        for (int j = 1; j <= NMAX; ++j) {
-            p += st;
-            x[j] = j < n ? *p : T(0);
-        }
-        lost.add(clamp_line<T, NMAX, false>(x, n, T(0), T(0), cf.c0, cf.c1, cf.c2, [&](int, T v) {
+        load_line<T, NMAX, false, 1>(x, n, [&]() { return next(p, st); });
+        lost.add(clamp_line<T, NMAX, false, 1>(x, n, T(0), T(0), cf.c0, cf.c1, cf.c2, [&](int, T v) {
             *w = v;
             w += st;
+            asm volatile("" : "+l"(w));
         }));
     }
     add_lost(lost, lost_out);
-}
-
-// one sweep of one FP32 line: n cells from p to w, element strides ps and ws
-// (both at the line's upwind end)
-template <int NMAX>
-__device__ __forceinline__ float sweep_line(const float *p, int ps, float *w, int ws, int n,
-                                            const LineCoef<float> &cf)
-{
-    float x[NMAX + 1];
-    x[0] = *p;
-#pragma unroll
-    for (int j = 1; j <= NMAX; ++j) {
-        p += ps;
-        x[j] = j < n ? *p : 0.f;
-    }
-    return clamp_line<float, NMAX, false>(x, n, 0.f, 0.f, cf.c0, cf.c1, cf.c2, [&](int, float v) {
-        *w = v;
-        w += ws;
-    });
 }
 
 // A block of G vx planes of a velocity cube (all of them: the whole cube) in
@@ -235,16 +221,60 @@ __device__ __forceinline__ void each_element(int count, int nz, F f)
     }
 }
 
+// one sweep of the block's lines along va, from src (IN) or the tile, into dst
+// (OUT) or the tile; which one it is is known at compile time, so that the tile
+// is addressed as shared memory (with one generic pointer for both a cell took
+// 35 instructions and the 24 x 28 x 26 kick 1.14 ms)
+template <int NMAX, bool IN, bool OUT>
+__device__ __forceinline__ void sweep_lines(const Block &B, int va, const float *src, float *dst, float *tile,
+                            const LineCoef<float> &c, Lost<float> &lost)
+{
+    constexpr int GR = NMAX <= 32 ? 4 : 1;
+    const int nz = B.nz, P = nz | 1, n = B.len(va), L = B.lines(va), neg = c.code & 1;
+    const int sp = neg ? -B.step(va, P) : B.step(va, P), sg = neg ? -B.step(va, nz) : B.step(va, nz);
+    for (int u = threadIdx.x; u < L; u += blockDim.x) {
+        const int a = B.first(va, u, P) + (neg ? (1 - n) * sp : 0);
+        const int g = IN || OUT ? B.first(va, u, nz) + (neg ? (1 - n) * sg : 0) : 0;
+        float x[NMAX + 1];
+        if constexpr (IN) {
+            const float *p = src + g;
+            load_line<float, NMAX, false, GR>(x, n, [&]() { return next(p, sg); });
+        } else {
+            int q = 4 * a;
+            load_line<float, NMAX, false, GR>(x, n, [&]() {
+                const float v = *reinterpret_cast<const float *>(reinterpret_cast<const char *>(tile) + q);
+                q += 4 * sp;
+                asm volatile("" : "+r"(q));
+                return v;
+            });
+        }
+        float *w = dst + g;
+        int r = 4 * a;
+        lost.add(clamp_line<float, NMAX, false, GR>(x, n, 0.f, 0.f, c.c0, c.c1, c.c2, [&](int, float v) {
+            if constexpr (OUT) {
+                *w = v;
+                w += sg;
+                asm volatile("" : "+l"(w));
+            } else {
+                *reinterpret_cast<float *>(reinterpret_cast<char *>(tile) + r) = v;
+                r += 4 * sp;
+                asm volatile("" : "+r"(r));
+            }
+        }));
+    }
+}
+
 // nsweeps consecutive sweeps first_axis, first_axis + 1, ... (mod 3) of a
 // block, from src (global, pitch nz) into dst.  The first sweep reads vx or vy
 // lines, and the last one writes them, straight from and to global memory
 // (coalesced along vz); vz rows, and sweeps that move by whole cells, go
 // through the tile.  Starts and ends with the tile free.
 template <int NMAX>
-__device__ void sweep_block(const Block &B, const float *src, float *dst, float *tile,
-                            const LineCoef<float> *cf, int nsweeps, int first_axis, Lost<float> &lost)
+__device__ __forceinline__ void sweep_block(const Block &B, const float *src, float *dst, float *tile,
+                                            const LineCoef<float> *cf, int nsweeps, int first_axis,
+                                            Lost<float> &lost)
 {
-    const int t = threadIdx.x, NT = blockDim.x, nz = B.nz, P = nz | 1, rows = B.g * B.ny;
+    const int nz = B.nz, P = nz | 1, rows = B.g * B.ny;
     auto whole = [&](int sw) { return (cf[sw].code >> 1) != 0; };
     const bool in = first_axis < 2 && !whole(0);
     if (!in) {
@@ -253,21 +283,20 @@ __device__ void sweep_block(const Block &B, const float *src, float *dst, float 
     }
     bool out = false;
     for (int sw = 0; sw < nsweeps; ++sw) {
-        const int va = (first_axis + sw) % 3, n = B.len(va), L = B.lines(va), st = B.step(va, P);
+        const int va = (first_axis + sw) % 3;
         const LineCoef<float> c = cf[sw];
-        const int neg = c.code & 1, sg = B.step(va, nz);
         out = sw == nsweeps - 1 && va < 2 && !whole(sw);
         if (whole(sw)) {
-            for (int u = t; u < L; u += NT) lost.add(kick_line_shifted(tile + B.first(va, u, P), st, n, c));
+            const int n = B.len(va), st = B.step(va, P);
+            for (int u = threadIdx.x; u < B.lines(va); u += blockDim.x)
+                lost.add(kick_line_shifted(tile + B.first(va, u, P), st, n, c));
+        } else if (sw == 0 && in) {
+            if (out) sweep_lines<NMAX, true, true>(B, va, src, dst, tile, c, lost);
+            else sweep_lines<NMAX, true, false>(B, va, src, dst, tile, c, lost);
+        } else if (out) {
+            sweep_lines<NMAX, false, true>(B, va, src, dst, tile, c, lost);
         } else {
-            for (int u = t; u < L; u += NT) {
-                const int a = B.first(va, u, P) + (neg ? (n - 1) * st : 0);
-                const int b = va < 2 ? B.first(va, u, nz) + (neg ? (n - 1) * sg : 0) : 0;
-                const float *p = sw == 0 && in ? src + b : tile + a;
-                float *w = out ? dst + b : tile + a;
-                const int ps = sw == 0 && in ? sg : st, ws = out ? sg : st;
-                lost.add(sweep_line<NMAX>(p, neg ? -ps : ps, w, neg ? -ws : ws, n, c));
-            }
+            sweep_lines<NMAX, false, false>(B, va, src, dst, tile, c, lost);
         }
         __syncthreads();
     }
@@ -287,7 +316,7 @@ __global__ void __launch_bounds__(512) k_kick_blocks(const float *src, float *ds
                                                     int nsweeps, int first_axis, int nx, int ny, int nz,
                                                     int G, long long np, double *lost_out)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+    extern __shared__ float tile[];
     __shared__ LineCoef<float> scf[6];
     const int per = (nx + G - 1) / G;
     Lost<float> lost;
@@ -299,8 +328,7 @@ __global__ void __launch_bounds__(512) k_kick_blocks(const float *src, float *ds
         __syncthreads();
         const Block B{nx - i0 < G ? nx - i0 : G, ny, nz};
         const long long off = (cell * nx + i0) * ny * (long long)nz;
-        sweep_block<NMAX>(B, src + off, dst + off, reinterpret_cast<float *>(smem_raw), scf, nsweeps,
-                          first_axis, lost);
+        sweep_block<NMAX>(B, src + off, dst + off, tile, scf, nsweeps, first_axis, lost);
     }
     add_lost(lost, lost_out);
 }
@@ -330,7 +358,10 @@ template <typename T>
 cudaError_t kick_lines_t(vp_ctx *c, const T *src, T *dst, const LineCoef<T> *coef, int va)
 {
     const int n = c->nv[va];
-    auto kern = n <= 16 ? k_kick_lines<T, 16> : (n <= 32 ? k_kick_lines<T, 32> : k_kick_lines<T, 64>);
+    auto kern = k_kick_lines<T, 64>;
+    if (n <= 16) kern = k_kick_lines<T, 16>;
+    else if (n <= 32) kern = k_kick_lines<T, 32>;
+    else if (n <= 48) kern = k_kick_lines<T, 48>;
     unsigned grid;
     const cudaError_t e = lines_grid(kern, c->np * (c->nvc / n), true, grid);
     if (e != cudaSuccess) return e;
@@ -350,7 +381,11 @@ cudaError_t kick_blocks(vp_ctx *c, const float *src, float *dst, const LineCoef<
     int threads = (lmax + 31) / 32 * 32;
     const int cap = smem > 110 * 1024 ? 512 : 256;
     if (threads > cap) threads = cap;
-    auto kern = c->maxnv <= 16 ? k_kick_blocks<16> : (c->maxnv <= 32 ? k_kick_blocks<32> : k_kick_blocks<64>);
+    auto kern = k_kick_blocks<64>;
+    if (c->maxnv <= 16) kern = k_kick_blocks<16>;
+    else if (c->maxnv <= 24) kern = k_kick_blocks<24>;
+    else if (c->maxnv <= 32) kern = k_kick_blocks<32>;
+    else if (c->maxnv <= 48) kern = k_kick_blocks<48>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
@@ -397,8 +432,10 @@ cudaError_t kick_lines_f32(vp_ctx *c, const float *src, float *dst, const LineCo
 template <typename T, bool PERIODIC>
 cudaError_t drift_lines_p(vp_ctx *c, const T *f, const LineCoef<T> *coef, const LinesGeom &g, T *fo)
 {
-    auto kern = g.n <= 16 ? k_drift_lines<T, 16, PERIODIC>
-                          : (g.n <= 32 ? k_drift_lines<T, 32, PERIODIC> : k_drift_lines<T, 64, PERIODIC>);
+    auto kern = k_drift_lines<T, 64, PERIODIC>;
+    if (g.n <= 16) kern = k_drift_lines<T, 16, PERIODIC>;
+    else if (g.n <= 32) kern = k_drift_lines<T, 32, PERIODIC>;
+    else if (g.n <= 48) kern = k_drift_lines<T, 48, PERIODIC>;
     unsigned grid;
     const cudaError_t e = lines_grid(kern, g.lines, drift_persistent<T, PERIODIC>(), grid);
     if (e != cudaSuccess) return e;
