@@ -141,4 +141,23 @@ __device__ __forceinline__ T clamp_line(const T (&x)[NMAX + 1], int n, T fm1, T 
     return phm;
 }
 
+// the same for FP32 lines of N cells known at compile time, in array order and
+// in place (outflow)
+template <int N, bool NEG>
+__device__ __forceinline__ float clamp_exact(float (&x)[N], float finf, float c0, float c1, float c2)
+{
+#define AT(j) x[NEG ? N - 1 - (j) : (j)]
+    float dm = AT(0), phm = 0.f;
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        const float f = AT(j), dp = (j + 1 < N ? AT(j + 1 < N ? j + 1 : 0) : 0.f) - f;
+        const float ph = clamp_flux(dm, f, dp, finf, c0, c1, c2);
+        AT(j) = (f - ph) + phm;
+        phm = ph;
+        dm = dp;
+    }
+#undef AT
+    return phm;
+}
+
 }  // namespace vpline

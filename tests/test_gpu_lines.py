@@ -100,6 +100,8 @@ def test_fp64_density_matches_oracle(n, nv):
     (37, 38, 39),       # whole cubes, one CTA per SM
     (63, 40, 30),       # blocks of vx planes, the last one not full
     (9, 64, 64), (50, 41, 37),
+    # vx planes of a compile-time size, the last block of planes not full
+    (37, 40, 40), (25, 48, 48), (19, 56, 56), (15, 64, 64),
 ])
 def test_fp32_steps_of_any_cube_match_oracle(nv, whole_cell):
     """Half kicks and the fused six-sweep kick (two steps); with whole_cell
@@ -137,3 +139,4 @@ def test_fp64_many_lines_match_oracle(n, space_bc):
     compare_sweep(w, 5, (0.25 * w.dv[2], -1.1 * w.dv[2]), n + 1)
     w = I.small_maxwell(n=(16, 8, 8), nv=(n, 5, 6), dtype="f64")
     compare_sweep(w, 3, (0.25 * w.dv[0], -1.1 * w.dv[0]), n + 2)
+
