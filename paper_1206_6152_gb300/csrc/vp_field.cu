@@ -407,7 +407,7 @@ template <class K>
 cudaError_t line_smem(K kernel, int B, int n, size_t &smem)
 {
     smem = (size_t)2 * B * (n + 1) * sizeof(double2);
-    if (smem <= 48 * 1024) return cudaSuccess;
+    if (smem + 1024 <= 48 * 1024) return cudaSuccess;
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
 }
 

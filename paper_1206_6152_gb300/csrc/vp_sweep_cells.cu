@@ -10,8 +10,8 @@
 // update reads its neighbour's flux from shared memory.  Any whole-cell shift.
 //
 // It pays while the lines do not fill the GPU's quadrants with a warp each (32
-// lanes x 4 quadrants x SMs = 19456 lines); above that the line kernels do less
-// work per cell.  128 x 128 cells (1D1V): x drift 88 -> 5 us, fused kick 140 ->
+// lanes x 4 quadrants x SMs = 19456 lines; the rules are below); above that the
+// line kernels do less work per cell.  128 x 128 cells (1D1V): x drift 88 -> 5 us, fused kick 140 ->
 // 10 us, and with the sweeps along periodic axes of one cell passed over a step
 // 254 -> 44 us.
 #include <cuda_runtime.h>
@@ -177,8 +177,14 @@ int threads_for(long long cells)
     return (int)(t > 512 ? 512 : t);
 }
 
-// lines enough for a warp on every quadrant of the GPU
-bool few_lines(const vp_ctx *c, long long lines) { return c->isdouble && lines < 128LL * vp_sm_count(); }
+// What a sweep along lines of n cells takes in units of one FP64 instruction of
+// the busiest quadrant: one thread per line, 7.3 instructions per cell and a
+// round of lines for every 32 lanes x 4 quadrants x SMs of them
+double lines_cost(const vp_ctx *c, int n)
+{
+    const long long round = 128LL * vp_sm_count(), lines = c->ncells / n;
+    return 7.3 * n * (double)((lines + round - 1) / round);
+}
 
 // lines per CTA of k_drift_cells: one while that gives at most four CTAs per
 // SM, and at most 4096 cells (64 KB of shared memory)
@@ -192,7 +198,13 @@ int cells_lines(const vp_ctx *c, int n)
 
 }  // namespace
 
-int vp_drift_cells_ok(const vp_ctx *c, int axis) { return few_lines(c, c->ncells / c->n[axis]); }
+// one thread per cell, 9 instructions (no difference is shared), where that is
+// the cheaper one: below 0.8 of a round of lines
+int vp_drift_cells_ok(const vp_ctx *c, int axis)
+{
+    const long long round = 128LL * vp_sm_count();
+    return c->isdouble && 9.0 * (double)((c->ncells + round - 1) / round) < lines_cost(c, c->n[axis]);
+}
 
 cudaError_t launch_drift_cells(vp_ctx *c, const void *f, int axis, const void *coef, void *fo)
 {
@@ -204,7 +216,7 @@ cudaError_t launch_drift_cells(vp_ctx *c, const void *f, int axis, const void *c
     const int vs = axis == 0 ? c->nv[1] * c->nv[2] : (axis == 1 ? c->nv[2] : 1);
     const size_t smem = (size_t)(2 * n * C + C) * sizeof(double);
     auto kern = c->periodic_space ? k_drift_cells<true> : k_drift_cells<false>;
-    if (smem > 48 * 1024) {
+    if (smem + 1024 > 48 * 1024) {      // (with the static part)
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
         if (e != cudaSuccess) return e;
     }
@@ -215,14 +227,21 @@ cudaError_t launch_drift_cells(vp_ctx *c, const void *f, int axis, const void *c
     return cudaGetLastError();
 }
 
-// cubes whose two buffers and line maxima fit in 96 KB
+// cubes whose two buffers and line maxima fit in 96 KB, where a cube's CTA (its
+// cells over 128 lanes, a round of cubes for every SM) is cheaper than one
+// thread per line: 128 cubes of 128 cells are by far, 4^3 cubes of 16^3 are not
+// (three steps 635 us against 362 us)
 int vp_kick_cells_ok(const vp_ctx *c)
 {
     int nmin = c->nv[0];
-    for (int a = 1; a < 3; ++a)
+    double lines = 0.0;
+    for (int a = 0; a < 3; ++a) {
         if (c->nv[a] < nmin) nmin = c->nv[a];
-    return few_lines(c, c->ncells / c->maxnv) &&
-           (2 * c->nvc + c->nvc / nmin) * sizeof(double) <= 96 * 1024;
+        lines += lines_cost(c, c->nv[a]);
+    }
+    const long long sms = vp_sm_count();
+    const double cells = 3 * 9.0 * (double)((c->np + sms - 1) / sms) * (double)((c->nvc + 127) / 128);
+    return c->isdouble && cells < lines && (2 * c->nvc + c->nvc / nmin) * sizeof(double) <= 96 * 1024;
 }
 
 cudaError_t launch_kick_cells(vp_ctx *c, const void *f, const void *ca, const void *cb, int nsweeps,
@@ -232,7 +251,7 @@ cudaError_t launch_kick_cells(vp_ctx *c, const void *f, const void *ca, const vo
     for (int a = 1; a < 3; ++a)
         if (c->nv[a] < nmin) nmin = c->nv[a];
     const size_t smem = (size_t)(2 * c->nvc + c->nvc / nmin) * sizeof(double);
-    if (smem > 48 * 1024) {
+    if (smem + 1024 > 48 * 1024) {      // (with the static part)
         const cudaError_t e = cudaFuncSetAttribute(k_kick_cells, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    96 * 1024);
         if (e != cudaSuccess) return e;

@@ -128,9 +128,9 @@ def test_fp32_steps_of_any_cube_match_oracle(nv, whole_cell):
 @pytest.mark.parametrize("space_bc", ["periodic", "outflow"])
 @pytest.mark.parametrize("n", [15, 18, 33, 64])
 def test_fp64_many_lines_match_oracle(n, space_bc):
-    """Lines enough to fill the GPU (21120 and more): one thread per line; the
-    tests above have few lines in FP64, which take one thread per cell."""
-    w = I.small_maxwell(n=(n, 4, 4), nv=(12, 11, 10), dtype="f64", space_bc=space_bc)
+    """Lines that fill the GPU in whole rounds (19008 of 19456 lanes): one thread
+    per line; the tests above have few lines in FP64, one thread per cell."""
+    w = I.small_maxwell(n=(n, 4, 4), nv=(12, 11, 9), dtype="f64", space_bc=space_bc)
     h, v = w.dx[0], max(abs(w.vlo[0]), abs(w.vhi[0]))
     compare_sweep(w, 0, (0.7 * h / v, -0.97 * h / v), n)
     if space_bc == "outflow":
@@ -140,3 +140,12 @@ def test_fp64_many_lines_match_oracle(n, space_bc):
     w = I.small_maxwell(n=(16, 8, 8), nv=(n, 5, 6), dtype="f64")
     compare_sweep(w, 3, (0.25 * w.dv[0], -1.1 * w.dv[0]), n + 2)
 
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("nv", [(13, 16, 14), (14, 14, 15), (18, 18, 18), (18, 18, 19)])
+def test_fp64_kick_at_the_shared_memory_limits(nv):
+    """Cubes whose buffers lie around the 48 KB of shared memory a launch has
+    without asking, and around the 96 KB up to which cubes take one thread per
+    cell."""
+    w = I.small_maxwell(n=(2, 2, 3), nv=nv, dtype="f64")
+    compare_sweep(w, 3, (0.25 * w.dv[0], -1.1 * w.dv[0]), sum(nv))
