@@ -333,8 +333,8 @@ __global__ void __launch_bounds__(256) k_functional_grad(T *__restrict__ lam_f,
 }
 
 // ---------------------------------------------------------------------------
-// register-line adjoint (line lengths 16/32/48/64, zero whole-cell shift):
-// the line of f, the output cotangent and the input cotangent live in
+// FP32 register-line adjoint (line lengths 16/32/48/64, zero whole-cell shift;
+// other lengths and FP64: vp_adjoint_lines.cu): the line of f, the output cotangent and the input cotangent live in
 // registers; the arms are evaluated with the same strict comparisons as
 // line_adjoint.  A line with a whole-cell shift is left untouched and
 // flagged for the generic kernel.
@@ -463,8 +463,7 @@ __global__ void __launch_bounds__(128) k_adjoint_fast(AdjArgs<T> A, LineGeom g, 
 int vp_adjoint_fast_ok(const vp_ctx *c, int axis)
 {
     const int n = axis < 3 ? c->n[axis] : c->nv[axis - 3];
-    if (c->isdouble) return n == 16;
-    return n == 16 || n == 32 || n == 48 || n == 64;
+    return !c->isdouble && (n == 16 || n == 32 || n == 48 || n == 64);
 }
 
 template <typename T, int N>
@@ -483,20 +482,15 @@ cudaError_t adjoint_fast_n(vp_ctx *c, const AdjArgs<T> &A, const LineGeom &g, di
     return cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t launch_adjoint_fast(vp_ctx *c, const AdjArgs<T> &A, const LineGeom &g, dim3 grid)
+cudaError_t launch_adjoint_fast(vp_ctx *c, const AdjArgs<float> &A, const LineGeom &g, dim3 grid)
 {
     cudaError_t e = cudaMemsetAsync(c->adj_flag, 0, sizeof(int), c->stream);
     if (e != cudaSuccess) return e;
-    if constexpr (sizeof(T) == 8) {
-        return adjoint_fast_n<T, 16>(c, A, g, grid);
-    } else {
-        switch (g.n) {
-        case 16: return adjoint_fast_n<T, 16>(c, A, g, grid);
-        case 32: return adjoint_fast_n<T, 32>(c, A, g, grid);
-        case 48: return adjoint_fast_n<T, 48>(c, A, g, grid);
-        default: return adjoint_fast_n<T, 64>(c, A, g, grid);
-        }
+    switch (g.n) {
+    case 16: return adjoint_fast_n<float, 16>(c, A, g, grid);
+    case 32: return adjoint_fast_n<float, 32>(c, A, g, grid);
+    case 48: return adjoint_fast_n<float, 48>(c, A, g, grid);
+    default: return adjoint_fast_n<float, 64>(c, A, g, grid);
     }
 }
 
@@ -570,9 +564,16 @@ cudaError_t sweep_adjoint_t(vp_ctx *c, const T *fin, T *lam, int axis, const Lin
     if (bc && !fast) {
         if ((e = launch_broadcast(c, bc, lam)) != cudaSuccess) return e;
     }
-    if (!fast && vp_adjoint_fast_ok(c, axis)) {
-        e = launch_adjoint_fast<T>(c, A, g, grid);
-        if (e != cudaSuccess) return e;
+    if constexpr (sizeof(T) == 4) {
+        if (!fast && vp_adjoint_fast_ok(c, axis)) {
+            if ((e = launch_adjoint_fast(c, A, g, grid)) != cudaSuccess) return e;
+            fast = true;
+        }
+    }
+    // every other line of 3 to 64 cells: 2 to 4 times faster than the routine below at
+    // each size measured (vp_adjoint_lines.cu); shorter and longer ones stay there
+    if (!fast && vp_adjoint_lines_ok(c, axis)) {
+        if ((e = launch_adjoint_lines(c, fin, lam, axis, coef, lam_g, dalpha_scale)) != cudaSuccess) return e;
         fast = true;
     }
     if (fast) {
