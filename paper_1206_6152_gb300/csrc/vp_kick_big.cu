@@ -6,7 +6,7 @@
 // a slab of vz planes, vz and vx inside a slab of vy planes, vy and vz inside
 // a slab of vx planes.  The fused kick K2^n K1^{n+1} (Sec. 2.1, Eq.
 // integration: vx vy vz vx vy vz) therefore runs as three passes over f,
-//   A: vx, vy   (K2 table)            on slabs of 8 vz planes
+//   A: vx, vy   (K2 table)            on slabs of 16 vz planes
 //   B: vz (K2), vx (K1)               on slabs of 8 vy planes
 //   C: vy, vz   (K1 table)            on slabs of 8 vx planes
 // and a single half kick (vx vy vz) as A followed by C without its first
@@ -16,15 +16,20 @@
 // between the two sweeps through a shared-memory tile.
 //
 //   A: the vx line pairs are read straight from global memory (a warp reads
-//      eight 32-byte row pieces per load), swept and written to the tile with
-//      the vy row index XOR-swizzled by the low bits of vx (so that both the
+//      four 64-byte row pieces per load), swept and written to the tile with
+//      the vy row index XOR-swizzled by the low bit of vx (so that both the
 //      vx and the vy line pairs move without bank conflicts), read back as
-//      vy line pairs, swept and stored straight to global memory.  The six
-//      slabs of a cube go to six CTAs that run at the same time, so every
-//      192-byte row is read from DRAM once.  (Slabs of 32-byte row pieces
-//      staged by asynchronous copies, cp.async or TMA, read three times
-//      their bytes from DRAM, whatever their L2 eviction policy; plain loads
-//      read them once.)
+//      vy line pairs, swept and stored straight to global memory.  The three
+//      slabs of a cube go to three CTAs that run at the same time, so every
+//      192-byte row is read from DRAM once, and each of them fetches a
+//      contiguous third of a cube of the next units into L2 while it sweeps.
+//      What bounds it: HBM, then requests to L2 of a quarter or half of a
+//      line.  Measured, one pass over 16 x 48 x 48 cubes (16.3 GB each way, 4.8 ms
+//      at 6.8 TB/s): 6.2 ms; 8.3 ms without the fetch; slabs of 8 planes (32-byte
+//      pieces, two CTAs per SM) 8.4 ms without and 9.3 ms with it.  (Slabs of
+//      32-byte row pieces staged by asynchronous copies, cp.async or TMA,
+//      read three times their bytes from DRAM, whatever their L2 eviction
+//      policy; plain loads read them once.)
 //   B: the slab (48 vx planes x 8 rows of 192 bytes) is prefetched into L2
 //      one unit ahead and copied into the tile with 16-byte cp.async
 //      copies; the vz sweep reads its row pairs from
@@ -61,9 +66,12 @@ struct Big3 {
     static constexpr int NU = N / S;           // slabs per cube
     static constexpr int NT = S * H;           // threads: one line pair each
     static constexpr int NC = N * N * N;
-    // tile of pass A: [vx][vy][8 vz], the vy row index XOR-swizzled with the
-    // low two bits of vx (conflict-free both as vx and as vy line pairs)
-    static constexpr int A_TILE = N * N * S;
+    // pass A: 16 vz planes per slab, one CTA per SM; tile [vx][vy][16 vz], the vy
+    // row index XOR-swizzled with the low bit of vx (conflict-free both as vx and
+    // as vy line pairs)
+    static constexpr int SA = 16;
+    static constexpr int NTA = SA * H;
+    static constexpr int A_TILE = N * N * SA;
     // tile of passes B and C: [slab plane][row][N], row pitch N + 4 (rows
     // read with 16-byte accesses without conflicts), plane pitch = 16 mod 32
     // banks (line pairs that straddle two planes stay conflict-free)
@@ -88,18 +96,18 @@ __device__ __forceinline__ void prefetch_l2(const void *p, unsigned bytes)
 __device__ __forceinline__ bool whole_cell(const LineCoef<float> &c) { return (c.code >> 1) != 0; }
 
 // ---------------------------------------------------------------------------
-// pass A: vx then vy on the slab of vz planes [8 s, 8 s + 8) of cube c; in
+// pass A: vx then vy on the slab of vz planes [16 s, 16 s + 16) of cube c; in
 // place or out of place
 // ---------------------------------------------------------------------------
 template <int N>
-__global__ void __launch_bounds__(Big3<N>::NT, 2) k_kick_pass_a(
+__global__ void __launch_bounds__(Big3<N>::NTA, 1) k_kick_pass_a(
     const float *src, const LineCoef<float> *__restrict__ coef, long long nunits,
     double *lost_out, float *dst)
 {
     typedef Big3<N> B;
-    constexpr int S = B::S, NU = B::NU, NC = B::NC;
+    constexpr int S = B::SA, NU = N / S, NC = B::NC;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    float *tile = reinterpret_cast<float *>(smem_raw);   // [vx][vy ^ (vx & 3)][8 vz]
+    float *tile = reinterpret_cast<float *>(smem_raw);   // [vx][vy ^ (vx & 1)][16 vz]
     __shared__ Acc<double> red[32];
     const int t = threadIdx.x, p = t % (S / 2), q = t / (S / 2);   // q: vy (sweep 1), vx (sweep 2)
     float lost = 0.f;
@@ -128,7 +136,7 @@ __global__ void __launch_bounds__(Big3<N>::NT, 2) k_kick_pass_a(
             continue;
         }
         // sweep 1: vx line pair at (vy = q, vz = k0 + 2p, + 1), from global
-        // memory (a warp reads eight 32-byte row pieces per load)
+        // memory (a warp reads four 64-byte row pieces per load)
         {
             const float *g = gs + q * N + k0 + 2 * p;
 #pragma unroll
@@ -139,14 +147,18 @@ __global__ void __launch_bounds__(Big3<N>::NT, 2) k_kick_pass_a(
             }
         }
         lost += sweep_pairs<N>(x, c1);
+        __syncthreads();        // the last unit's vy lines are read
 #pragma unroll
         for (int i = 0; i < N; ++i)
-            *reinterpret_cast<float2 *>(tile + i * N * S + ((q ^ (i & 3)) * S) + 2 * p) = x[i];
+            *reinterpret_cast<float2 *>(tile + i * N * S + ((q ^ (i & (32 / S - 1))) * S) + 2 * p) = x[i];
         __syncthreads();
+        // a third of a cube of the next units into L2
+        const long long un = u + gridDim.x;
+        if (t < 8 && un < nunits) prefetch_l2(src + un * (NC / NU) + t * (NC / NU / 8), NC / NU / 2);
         // sweep 2: vy line pair at (vx = q, vz = k0 + 2p, + 1)
 #pragma unroll
         for (int j = 0; j < N; ++j)
-            x[j] = *reinterpret_cast<const float2 *>(tile + q * N * S + ((j ^ (q & 3)) * S) + 2 * p);
+            x[j] = *reinterpret_cast<const float2 *>(tile + q * N * S + ((j ^ (q & (32 / S - 1))) * S) + 2 * p);
         lost += sweep_pairs<N>(x, c2);
         {
             float *g = gd + q * N * N + k0 + 2 * p;
@@ -157,7 +169,6 @@ __global__ void __launch_bounds__(Big3<N>::NT, 2) k_kick_pass_a(
                 asm volatile("" : "+l"(g));
             }
         }
-        __syncthreads();        // the tile is rewritten by the next unit
     }
     Acc<double> a;
     a.add((double)lost);
@@ -399,8 +410,8 @@ cudaError_t launch_kick_big3(vp_ctx *c, float *f, const LineCoef<float> *ca,
     const size_t smem_bc = (size_t)B::BC_TILE * sizeof(float);
     cudaEvent_t *ev = c->kick_pass_ev;
     if (ev && (e = cudaEventRecord(ev[0], c->stream)) != cudaSuccess) return e;
-    if ((e = persistent_grid(k_kick_pass_a<N>, B::NT, smem_a, nunits, grid)) != cudaSuccess) return e;
-    k_kick_pass_a<N><<<grid, B::NT, smem_a, c->stream>>>(f, ca, nunits, &c->sc->lost, fo);
+    if ((e = persistent_grid(k_kick_pass_a<N>, B::NTA, smem_a, c->np * (N / B::SA), grid)) != cudaSuccess) return e;
+    k_kick_pass_a<N><<<grid, B::NTA, smem_a, c->stream>>>(f, ca, c->np * (N / B::SA), &c->sc->lost, fo);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (ev && (e = cudaEventRecord(ev[1], c->stream)) != cudaSuccess) return e;
     if (nsweeps == 2) {             // vx and vy only: pass A
