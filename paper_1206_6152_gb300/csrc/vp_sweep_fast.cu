@@ -284,6 +284,11 @@ __global__ void __launch_bounds__(KickCube<N>::NT) k_kick_fast(float *__restrict
 // The fused kick pass K2^n K1^{n+1}: six sweeps vx vy vz vx vy vz of every
 // cube (coefficient tables ca for the first three, cb for the last three),
 // in place or into fo.
+// What bounds it: with one CTA per SM (the cube fills shared memory) the shared-memory
+// phases (twelve passes over the cube) and the FP32 phases, 41 % of the peak each,
+// hardly overlap.  For N = 32 the next cube's lines are loaded before this one is
+// copied out: 32^6 3.93 -> 3.86 ms (its bytes take 1.26 ms at 6.8 TB/s), 16^3 x 32^3
+// 519 -> 507 us; 32^3 x 16^3 444 -> 451 us, so not for N = 16, with several CTAs per SM.
 template <int N>
 __global__ void __launch_bounds__(KickCube<N>::NT) k_kick6(float *__restrict__ f,
                                                          const LineCoef<float> *__restrict__ ca,
@@ -299,22 +304,23 @@ __global__ void __launch_bounds__(KickCube<N>::NT) k_kick6(float *__restrict__ f
     const int t = threadIdx.x;
     float lost = 0.f;
     int par = 0;
+    constexpr bool EARLY = N > 16;
+    float2 x[N];
+    if (EARLY && blockIdx.x < np) load_pairs<N, true>(f + blockIdx.x * (long long)NC, 0, t, x);
     for (long long cell = blockIdx.x; cell < np; cell += gridDim.x, par ^= 1) {
         float *g = f + cell * (long long)NC;
         float *go = fo + cell * (long long)NC;
-        if (t < 4) {
-            const long long nx = cell + gridDim.x;
-            if (nx < np) prefetch_l2(f + nx * NC + t * (NC / 4), NC);
-        }
+        const long long nx = cell + gridDim.x;
+        if (t < 4 && nx < np) prefetch_l2(f + nx * NC + t * (NC / 4), NC);
         if (t < 6) scf[par][t] = (t < 3 ? ca : cb)[cell * 3 + t % 3];
-        float2 x[N];
-        load_pairs<N, true>(g, 0, t, x);
+        if (!EARLY) load_pairs<N, true>(g, 0, t, x);
         __syncthreads();
         bool shifted = false;
 #pragma unroll
         for (int sw = 0; sw < 6; ++sw) shifted |= (scf[par][sw].code >> 1) != 0;
         if (shifted) {
             lost += kick_cube_shifted<N>(g, go, cube, scf[par], 6, 0);
+            if (EARLY && nx < np) load_pairs<N, true>(f + nx * NC, 0, t, x);
             continue;
         }
         lost += sweep_pairs<N>(x, scf[par][0]);
@@ -339,6 +345,8 @@ __global__ void __launch_bounds__(KickCube<N>::NT) k_kick6(float *__restrict__ f
         load_rows<N, false>(cube, t, x);
         lost += sweep_pairs<N>(x, scf[par][5]);
         store_rows<N, false>(cube, t, x);
+        // the next cube's loads are under way while this one is copied out
+        if (EARLY && nx < np) load_pairs<N, true>(f + nx * NC, 0, t, x);
         __syncwarp();
         copy_out_rows<N>(go, cube, t >> 5, t & 31);
     }
