@@ -526,18 +526,32 @@ __device__ __forceinline__ long long unit_to_v(long long L, const DriftGeom &g)
     return L * 2;
 }
 
-// RHO: the per-thread compensated density sums of the N cells of the line
-// live in shared memory (slot j of thread t at j * 128 + t: conflict-free),
-// which keeps the kernel at 128 registers (16 warps per SM)
+// RHO: the compensated density sums of the N cells of the line, one per pair of
+// velocity cells the thread (or, for lines of more than 32 cells, the two lanes of the
+// pair) visits, live in shared memory (slot j of pair q at 128 j + q, or at q ^ 8 for odd
+// j of the lanes' form: conflict-free); the rows of the CTA's next lines are fetched into L2.
+// What bounds it: HBM; with the density, lines of 48 and 64 in pairs (255 registers, 8
+// warps per SM) were bound by latency, so these take one line per thread (16 warps;
+// the lanes of a pair exchange cells so that each sum is formed in the pairs' order).
+// Measured, x drift: 64 x 32^2 of 32^3 cells (2.5 ms at 6.8 TB/s) 3.90 -> 3.46 ms, 64 x 16^2
+// 1.40 -> 0.95 ms, 48 x 16^2 of 48^3 2.16 -> 2.02 ms; the fetch alone 32^6 1.48 -> 1.45 ms,
+// 16^3 of 32^3 234 -> 222 us.  Without the density pairs stay: single lines of 48 were
+// slower (y, z drift of 16 x 48^2 of 48^3 5.1 -> 5.3 ms), as were lines of 64 (804 -> 873 us).
+template <int N, bool RHO>
+constexpr bool drift_single = RHO && N > 32;      // one line per thread, not a pair
+template <int N, bool RHO>
+constexpr int drift_threads = drift_single<N, RHO> ? 256 : 128;
+
 template <int N, bool PERIODIC, bool RHO>
-__global__ void __launch_bounds__(128, N <= 32 ? 4 : 1) k_drift_fast(const float *__restrict__ f,
+__global__ void __launch_bounds__(drift_threads<N, RHO>, N <= 32 ? 4 : (RHO ? 2 : 1)) k_drift_fast(const float *__restrict__ f,
                                                                const LineCoef<float> *__restrict__ coef,
                                                                DriftGeom g, double *__restrict__ rho_part,
                                                                double *lost_out, float *__restrict__ fo)
 {
     __shared__ Acc<double> red[32];
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    Acc<float> *sacc = reinterpret_cast<Acc<float> *>(smem_raw) + threadIdx.x;   // slot j: sacc[j * 128]
+    Acc<float> *sacc = reinterpret_cast<Acc<float> *>(smem_raw);
+    const int t = threadIdx.x;
     const int o = blockIdx.y;
     const long long base_cell = (long long)(o / g.od) * g.m1 + (long long)(o % g.od) * g.m2;
     const long long gstride = g.cell_stride * g.nvc;
@@ -546,58 +560,135 @@ __global__ void __launch_bounds__(128, N <= 32 ? 4 : 1) k_drift_fast(const float
     const long long u0 = (long long)blockIdx.x * g.per_part;
     long long u1 = u0 + g.per_part;
     if (u1 > g.nunits) u1 = g.nunits;
-    if constexpr (RHO) {
-#pragma unroll
-        for (int j = 0; j < N; ++j) sacc[j * 128] = Acc<float>();
-    }
+    // x sweeps: row t of the CTA's next 128 pairs into L2
+    auto fetch_next = [&](long long L) {
+        if (RHO && t < N && L + 128 < u1) {
+            const long long nu = u1 - L - 128 < 128 ? u1 - L - 128 : 128;
+            const float *p = fb + t * gstride + (L + 128) * 2;
+            if ((((size_t)p | (size_t)(nu * 8)) & 15) == 0) prefetch_l2(p, (unsigned)(nu * 8));
+        }
+    };
     float lost = 0.f;
-    for (long long L = u0 + threadIdx.x; L < u1; L += blockDim.x) {
-        const long long v = unit_to_v(L, g);
-        float2 x[N];
-        // the line's addresses are stepped through an opaque register: the
-        // compiler would otherwise keep all 2 N of them live across the update
-        const float *p = fb + v;
-#pragma unroll
-        for (int j = 0; j < N; ++j) {
-            x[j] = *reinterpret_cast<const float2 *>(p);
-            p += gstride;
-            asm volatile("" : "+l"(p));
-        }
-        const int via = (int)((v / g.va_stride) % g.va_n);
-        const int vib = (int)(((v + 1) / g.va_stride) % g.va_n);
-        lost += drift_pair<N, PERIODIC>(x, coef[via], coef[vib]);
-        float *q = ob + v;
-#pragma unroll
-        for (int j = 0; j < N; ++j) {
-            *reinterpret_cast<float2 *>(q) = x[j];
-            q += gstride;
-            asm volatile("" : "+l"(q));
-        }
+    if constexpr (!drift_single<N, RHO>) {
+        sacc += t;
         if constexpr (RHO) {
 #pragma unroll
+            for (int j = 0; j < N; ++j) sacc[j * 128] = Acc<float>();
+        }
+        for (long long L = u0 + t; L < u1; L += 128) {
+            const long long v = unit_to_v(L, g);
+            fetch_next(L - t);
+            float2 x[N];
+            // the line's addresses are stepped through an opaque register: the
+            // compiler would otherwise keep all 2 N of them live across the update
+            const float *p = fb + v;
+#pragma unroll
             for (int j = 0; j < N; ++j) {
-                Acc<float> a = sacc[j * 128];
-                a.add(x[j].x);
-                a.add(x[j].y);
-                sacc[j * 128] = a;
+                x[j] = *reinterpret_cast<const float2 *>(p);
+                p += gstride;
+                asm volatile("" : "+l"(p));
+            }
+            const int via = (int)((v / g.va_stride) % g.va_n);
+            const int vib = (int)(((v + 1) / g.va_stride) % g.va_n);
+            lost += drift_pair<N, PERIODIC>(x, coef[via], coef[vib]);
+            float *q = ob + v;
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                *reinterpret_cast<float2 *>(q) = x[j];
+                q += gstride;
+                asm volatile("" : "+l"(q));
+            }
+            if constexpr (RHO) {
+#pragma unroll
+                for (int j = 0; j < N; ++j) {
+                    Acc<float> a = sacc[j * 128];
+                    a.add(x[j].x);
+                    a.add(x[j].y);
+                    sacc[j * 128] = a;
+                }
             }
         }
-    }
-    if constexpr (RHO) {
-        // per-x reduction over the CTA, written as one partial per (part, cell)
+        if constexpr (RHO) {
+            // per-x reduction over the CTA, written as one partial per (part, cell)
 #pragma unroll
-        for (int j = 0; j < N; ++j) {
-            Acc<float> a = block_merge(sacc[j * 128], reinterpret_cast<Acc<float> *>(red));
-            if (threadIdx.x == 0)
-                rho_part[(long long)blockIdx.x * g.np + base_cell + j * g.cell_stride] = a.value();
+            for (int j = 0; j < N; ++j) {
+                Acc<float> a = block_merge(sacc[j * 128], reinterpret_cast<Acc<float> *>(red));
+                if (t == 0) rho_part[(long long)blockIdx.x * g.np + base_cell + j * g.cell_stride] = a.value();
+                __syncthreads();
+            }
+        }
+    } else {
+        // one line per thread, the lanes 2 i and 2 i + 1 a pair
+        const int pr = t >> 1, odd = t & 1;
+        if constexpr (RHO) {
+            for (int e = t; e < N * 128; e += 256) sacc[e] = Acc<float>();
             __syncthreads();
+        }
+        for (long long L0 = u0; L0 < u1; L0 += 128) {
+            const bool active = L0 + pr < u1;
+            const long long v = unit_to_v(active ? L0 + pr : u0, g) + odd;     // (u0: no load)
+            fetch_next(L0);
+            float x[N];
+            const float *p = fb + v;
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                x[j] = active ? *p : 0.f;
+                p += gstride;
+                asm volatile("" : "+l"(p));
+            }
+            const LineCoef<float> cf = coef[(int)((v / g.va_stride) % g.va_n)];
+            const float out = update_line<float, N, PERIODIC>(x, weights_one<float>(cf, line_max(x)), cf.code & 1);
+            if (active) {
+                lost += out;
+                float *q = ob + v;
+#pragma unroll
+                for (int j = 0; j < N; ++j) {
+                    *q = x[j];
+                    q += gstride;
+                    asm volatile("" : "+l"(q));
+                }
+            }
+            if constexpr (RHO) {
+                // cells j, j + 1 of the pair: the even lane adds those of j, the odd
+                // lane those of j + 1, the even line's value first
+#pragma unroll
+                for (int j = 0; j < N; j += 2) {
+                    const float other = __shfl_xor_sync(0xffffffffu, odd ? x[j] : x[j + 1], 1);
+                    Acc<float> *s = sacc + (j + odd) * 128 + (pr ^ (odd << 3));
+                    if (active) {
+                        Acc<float> a = *s;
+                        a.add(odd ? other : x[j]);
+                        a.add(odd ? x[j + 1] : other);
+                        *s = a;
+                    }
+                }
+            }
+        }
+        if constexpr (RHO) {
+            // as block_merge over the 128 pairs, two slots at a time
+            Acc<float> *part = reinterpret_cast<Acc<float> *>(red) + 4 * (t >> 7);
+            const int lane = t & 31, warp = (t >> 5) & 3;
+            for (int j = t >> 7; j < N; j += 2) {
+                __syncthreads();
+                Acc<float> a = sacc[j * 128 + ((t & 127) ^ ((j & 1) << 3))];
+                for (int d = 16; d > 0; d >>= 1) a.shfl_merge(d);
+                if (lane == 0) part[warp] = a;
+                __syncthreads();
+                if (warp == 0) {
+                    Acc<float> b;
+                    if (lane < 4) b = part[lane];
+                    for (int d = 16; d > 0; d >>= 1) b.shfl_merge(d);
+                    if (lane == 0)
+                        rho_part[(long long)blockIdx.x * g.np + base_cell + j * g.cell_stride] = b.value();
+                }
+            }
         }
     }
     if (!PERIODIC) {
         Acc<double> a;
         a.add((double)lost);
         a = block_merge(a, red);
-        if (threadIdx.x == 0 && a.value() != 0.0) atomicAdd(lost_out, a.value());
+        if (t == 0 && a.value() != 0.0) atomicAdd(lost_out, a.value());
     }
 }
 
@@ -818,10 +909,10 @@ cudaError_t drift_fast_n(vp_ctx *c, float *f, int axis, const LineCoef<float> *c
         auto kern = c->periodic_space ? k_drift_fast<N, true, true> : k_drift_fast<N, false, true>;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)racc);
         if (e != cudaSuccess) return e;
-        kern<<<grid, 128, racc, c->stream>>>(f, coef, g, rho_part, lost, o);
+        kern<<<grid, drift_threads<N, true>, racc, c->stream>>>(f, coef, g, rho_part, lost, o);
     } else {
         auto kern = c->periodic_space ? k_drift_fast<N, true, false> : k_drift_fast<N, false, false>;
-        kern<<<grid, 128, 0, c->stream>>>(f, coef, g, rho_part, lost, o);
+        kern<<<grid, drift_threads<N, false>, 0, c->stream>>>(f, coef, g, rho_part, lost, o);
     }
     return cudaGetLastError();
 }
