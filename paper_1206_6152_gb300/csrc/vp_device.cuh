@@ -25,6 +25,37 @@ __device__ __forceinline__ float vmin(float a, float b) { return fminf(a, b); }
 __device__ __forceinline__ float vmax(float a, float b) { return fmaxf(a, b); }
 
 // ---------------------------------------------------------------------------
+// n / d for 0 <= n < 2^31 by a divisor known on the host (Granlund & Montgomery,
+// "Division by invariant integers using multiplication", 1994): a multiplication,
+// an addition and a shift, where a 64-bit division takes about a hundred
+// instructions, as many as four to eight cells of a sweep.
+// ---------------------------------------------------------------------------
+struct FastDiv {
+    unsigned m = 1, s = 0;      // (d = 1)
+    FastDiv() = default;
+    explicit FastDiv(unsigned d)
+    {
+        while ((1ull << s) < d) ++s;
+        m = (unsigned)(((1ull << 32) * ((1ull << s) - d)) / d + 1);
+    }
+    __device__ __forceinline__ unsigned operator()(unsigned n) const { return (__umulhi(m, n) + n) >> s; }
+};
+
+// index along an axis of velocity cell v: (v / stride) % n
+struct VelIndex {
+    FastDiv by_stride, by_n;
+    int stride = 1, n = 1;
+    VelIndex() = default;
+    VelIndex(int stride_, int n_) : by_stride(stride_), by_n(n_), stride(stride_), n(n_) {}
+    __device__ __forceinline__ int operator()(long long v) const
+    {
+        if (v >= (1LL << 31)) return (int)((v / stride) % n);
+        const unsigned a = by_stride((unsigned)v);
+        return (int)(a - by_n(a) * (unsigned)n);
+    }
+};
+
+// ---------------------------------------------------------------------------
 // PFC partial flux of cell j (Sec. 2.1): the integral of the third-order
 // reconstruction over the fraction beta of cell j that crosses its downwind
 // face, in units of the cell average.  The slope corrector of Filbet,

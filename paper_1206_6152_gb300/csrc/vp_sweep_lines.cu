@@ -9,7 +9,10 @@
 //    load).  Scalar lines, not packed pairs, so that each lane reads its own
 //    direction.  FP32: bound by HBM; 20 x 18 x 22 positions of 24 x 28 x 26
 //    velocity cells 0.30 -> 0.21 ms a sweep (5.3 TB/s) against the shared-memory
-//    kernel.  FP64: at the FP64 pipe's rate (7.3 instructions per cell counted,
+//    kernel.  Indices by multiplication (FastDiv): with 64-bit divisions, about a
+//    hundred instructions each, lines of 4 to 20 cells were bound by issue (x drift
+//    of 4 x 64^2 of 32^3 cells 1.65 -> 1.36 ms, 8 x 8 x 4 of 48^3, z 95 -> 80, x 60 ->
+//    53 us).  FP64: at the FP64 pipe's rate (7.3 instructions per cell counted,
 //    74 cycles each per quadrant's warp); 20 x 18 x 22 of the same 1.48 -> 0.86
 //    ms, and FP64 lines of 16 and 32 go through here as well: the saturating
 //    form takes 9 FP64 instructions and a reciprocal per line, and the z drift
@@ -101,7 +104,8 @@ struct LinesGeom {
     int od;                    // outer index o -> first cell: (o / od) m1 + (o % od) m2
     long long m1, m2;
     int nvc;                   // velocity cells per spatial cell
-    int va_stride, va_n;       // velocity index along the axis: (v / va_stride) % va_n
+    FastDiv by_nvc, by_od;
+    VelIndex vel;              // velocity index along the axis
     long long lines;           // outer indices times nvc
 };
 
@@ -119,10 +123,11 @@ __global__ void __launch_bounds__(128) k_drift_lines(const T *f, const LineCoef<
     Lost<T> lost;
     for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < g.lines;
          q += (long long)gridDim.x * blockDim.x) {
-        const int o = (int)(q / g.nvc), v = (int)(q - (long long)o * g.nvc);
-        const LineCoef<T> cf = coef[(v / g.va_stride) % g.va_n];
+        const int o = q < (1LL << 31) ? (int)g.by_nvc((unsigned)q) : (int)(q / g.nvc);
+        const int v = (int)(q - (long long)o * g.nvc), oh = (int)g.by_od((unsigned)o);
+        const LineCoef<T> cf = coef[g.vel(v)];
         const bool neg = cf.code & 1;
-        const long long off = ((o / g.od) * g.m1 + (o % g.od) * g.m2) * g.nvc + v +
+        const long long off = (oh * g.m1 + (o - oh * g.od) * g.m2) * g.nvc + v +
                               (neg ? (n - 1) * step : 0);
         const long long st = neg ? -step : step;
         T x[NMAX + 1];
@@ -584,8 +589,9 @@ cudaError_t drift_lines_t(vp_ctx *c, const T *f, int axis, const LineCoef<T> *co
         g.od = 1; g.m1 = c->n[2]; g.m2 = 0;
     }
     g.nvc = (int)c->nvc;
-    g.va_stride = axis == 0 ? c->nv[1] * c->nv[2] : (axis == 1 ? c->nv[2] : 1);
-    g.va_n = c->nv[axis];
+    g.by_nvc = FastDiv(g.nvc);
+    g.by_od = FastDiv(g.od);
+    g.vel = VelIndex(axis == 0 ? c->nv[1] * c->nv[2] : (axis == 1 ? c->nv[2] : 1), c->nv[axis]);
     g.lines = c->np / g.n * c->nvc;
     const LineCoef<T> *cf = coef + (size_t)axis * c->maxnv;
     return c->periodic_space ? drift_lines_p<T, true>(c, f, cf, g, fo)
