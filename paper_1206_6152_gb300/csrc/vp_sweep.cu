@@ -365,8 +365,16 @@ __global__ void k_coef_step(LineCoef<T> *__restrict__ kick, const double *__rest
 }
 
 // ---------------------------------------------------------------------------
-// rho(x) = dv^3 sum_v f (Sec. 2.2), compensated: one CTA per velocity cube
+// rho(x) = dv^3 sum_v f (Sec. 2.2), compensated: one CTA per velocity cube.
+// Bound by HBM where CTAs fill the SMs, else by the latency of each thread's loads:
+// U > 1 takes U of them at a time, in the same order of additions (same bits).
+// Measured, U = 8 against 1: 2^3 of 64^3 cells 66 -> 37 us, 8 x 8 x 4 of 48^3 61 -> 37 us;
+// with one value per load (cubes that are no multiple of 4) 20 x 18 x 22 of 25 x 27 x
+// 23 212 -> 124 us, 3 x 2 x 2 of 31 x 33 x 47 53 -> 17 us.  Where the SMs are full anyway U = 1
+// is as good or better (4 x 64^2 of 32^3 342 against 356 us, 60000 cubes of 5^3 69
+// against 93 us).
 // ---------------------------------------------------------------------------
+template <int U>
 __global__ void __launch_bounds__(256) k_density(const float *__restrict__ f, long long np, int nvc,
                                                 double dvol, double *__restrict__ rho)
 {
@@ -379,18 +387,34 @@ __global__ void __launch_bounds__(256) k_density(const float *__restrict__ f, lo
             // memory-level parallelism, merged at the end
             Acc<float> b, c2, d;
             const float4 *q4 = reinterpret_cast<const float4 *>(q);
-            for (int e = threadIdx.x; e < nvc / 4; e += blockDim.x) {
-                const float4 v = q4[e];
+            auto add = [&](const float4 &v) {
                 a.add(v.x);
                 b.add(v.y);
                 c2.add(v.z);
                 d.add(v.w);
+            };
+            int e = threadIdx.x;
+            for (; U > 1 && e + (U - 1) * (int)blockDim.x < nvc / 4; e += U * blockDim.x) {
+                float4 v[U];
+#pragma unroll
+                for (int i = 0; i < U; ++i) v[i] = q4[e + i * blockDim.x];
+#pragma unroll
+                for (int i = 0; i < U; ++i) add(v[i]);
             }
+            for (; e < nvc / 4; e += blockDim.x) add(q4[e]);
             a.merge(b);
             c2.merge(d);
             a.merge(c2);
         } else {
-            for (int e = threadIdx.x; e < nvc; e += blockDim.x) a.add(q[e]);
+            int e = threadIdx.x;
+            for (; U > 1 && e + (U - 1) * (int)blockDim.x < nvc; e += U * blockDim.x) {
+                float v[U];
+#pragma unroll
+                for (int i = 0; i < U; ++i) v[i] = q[e + i * blockDim.x];
+#pragma unroll
+                for (int i = 0; i < U; ++i) a.add(v[i]);
+            }
+            for (; e < nvc; e += blockDim.x) a.add(q[e]);
         }
         a = block_merge(a, red);
         if (threadIdx.x == 0) rho[cell] = a.value() * dvol;
@@ -680,8 +704,11 @@ cudaError_t launch_density(vp_ctx *c, const void *f, double *rho)
     const long long cap = (long long)sm_count() * 8;
     long long grid = c->np < cap ? c->np : cap;
     if (!c->isdouble) {
-        k_density<<<(unsigned)grid, 256, 0, c->stream>>>((const float *)f, c->np, (int)c->nvc, c->dvol_v,
-                                                         rho);
+        // (a thread has at least 8 loads; four values a load: only where CTAs are few,
+        // 1280 cubes of 32^3 52 -> 37 us, 7920 of 24 x 28 x 26 109 -> 111)
+        const bool batch = c->nvc % 4 ? c->nvc >= 2048 : c->nvc >= 8192 && c->np < 2 * cap;
+        auto kern = batch ? k_density<8> : k_density<1>;
+        kern<<<(unsigned)grid, 256, 0, c->stream>>>((const float *)f, c->np, (int)c->nvc, c->dvol_v, rho);
     } else if (c->np >= 16LL * sm_count() || c->nvc <= 512) {
         // (few small cubes: one warp per CTA, so that the warps spread over the SMs)
         const int per = c->np >= 16LL * sm_count() ? 8 : 1;
