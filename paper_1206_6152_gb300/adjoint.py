@@ -84,10 +84,10 @@ class _Trajectory(torch.autograd.Function):
         sim: VlasovPoisson = ctx.sim
         f = sim.f
         fbytes = f.numel() * f.element_size()
-        if f.is_cuda:
-            # the adjoint's scratch states are allocated by the library, outside
-            # torch's caching allocator: blocks torch keeps cached would not be
-            # available to it
+        # the adjoint's scratch states (nine at most) are allocated by the library,
+        # outside torch's caching allocator: blocks torch keeps cached would not be
+        # available to it, and go back to the device where it might run short
+        if f.is_cuda and _free_bytes(f.device) < (ctx.every + 16) * fbytes:
             torch.cuda.empty_cache()
         with torch.no_grad():
             lam_f = ctx.lam_f
@@ -106,11 +106,14 @@ class _Trajectory(torch.autograd.Function):
                     sim.set_accel(gc)
                     # every step-start state is kept, so the steps run one
                     # call each (inside a fused body the state between two
-                    # steps is never in memory)
+                    # steps is never in memory); the first is the checkpoint
+                    # itself, the last the context's own f
                     states = []
                     for n in range(n0, n1):
-                        states.append((f.clone(), sim.field()[2]))
-                        if n + 1 < n1:          # f^{n1} is not needed
+                        last = n + 1 == n1      # f^{n1} is not needed
+                        fs = f if last else (fc if n == n0 and fc.device == f.device else f.clone())
+                        states.append((fs, sim.field()[2]))
+                        if not last:
                             sim.step(1)
                     for fs, gs in reversed(states):
                         sim.adjoint_step(fs, gs, lam_f, lam_g)
