@@ -55,6 +55,30 @@ struct VelIndex {
     }
 };
 
+// Blocks of the fused y and z drifts: block b = (x plane, chunk of vc velocity cells of one
+// vz row), chunks fastest.
+struct YZBlocks {
+    long long nvb = 1;          // chunks per x plane (below 2^31)
+    FastDiv by_nvb, by_row, by_nvy;
+    int row = 1, nvy = 1;       // chunks per vz row
+    YZBlocks(long long nvc, int nvy_, int nvz, int vc)
+        : nvb(nvc / vc), by_nvb((unsigned)(nvc / vc)), by_row(nvz / vc), by_nvy(nvy_), row(nvz / vc), nvy(nvy_)
+    {
+    }
+    __device__ __forceinline__ void split(long long b, long long &x, unsigned &chunk) const
+    {
+        x = b < (1LL << 31) ? by_nvb((unsigned)b) : b / nvb;
+        chunk = (unsigned)(b - x * nvb);
+    }
+    // vy index of a chunk and its first vz index in units of chunks
+    __device__ __forceinline__ void velocity(unsigned chunk, int &vy, int &vzc) const
+    {
+        const unsigned r = by_row(chunk);
+        vzc = (int)(chunk - r * (unsigned)row);
+        vy = (int)(r - by_nvy(r) * (unsigned)nvy);
+    }
+};
+
 // ---------------------------------------------------------------------------
 // PFC partial flux of cell j (Sec. 2.1): the integral of the third-order
 // reconstruction over the fraction beta of cell j that crosses its downwind

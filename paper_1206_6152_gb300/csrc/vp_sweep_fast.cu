@@ -703,7 +703,10 @@ __global__ void __launch_bounds__(drift_threads<N, RHO>, N <= 32 ? 4 : (RHO ? 2 
 // sweeps.  The chunk lies inside one vz
 // row, so every y line of the CTA has the same v_y; the z lines of a pair
 // differ in v_z (two coefficients, two scalar lines where the pair
-// straddles the sign change of v_z).
+// straddles the sign change of v_z).  Bound by HBM; its block and velocity indices
+// are multiplications (YZBlocks), as nine 64-bit divisions a block took almost as
+// many instructions as the sweeps: 32^6 1.60 -> 1.52 ms (1.26 ms at 6.8 TB/s), 16^3 of
+// 32^3 262 -> 252 us, 64 x 32^2 of 32^3 3.24 -> 3.08 ms.
 // ---------------------------------------------------------------------------
 template <int N>
 struct DriftYZ {
@@ -718,7 +721,7 @@ template <int N, bool PERIODIC>
 __global__ void __launch_bounds__(DriftYZ<N>::NT, 2) k_drift_yz(const float *__restrict__ f,
                                                               const LineCoef<float> *__restrict__ cz,
                                                               const LineCoef<float> *__restrict__ cy,
-                                                              long long nvc, int nvy, int nvz,
+                                                              long long nvc, YZBlocks g,
                                                               long long nblocks, double *lost_out,
                                                               float *__restrict__ fo)
 {
@@ -727,14 +730,15 @@ __global__ void __launch_bounds__(DriftYZ<N>::NT, 2) k_drift_yz(const float *__r
     float *tile = reinterpret_cast<float *>(smem_raw);
     __shared__ Acc<double> red[32];
     const int t = threadIdx.x, vp = t % H, r = t / H;    // r: y in the z sweep, z in the y sweep
-    const long long nvb = nvc / VC;                      // velocity blocks per x plane
     float lost = 0.f;
-    // block b = (x plane b / nvb, velocity cells [VC (b % nvb), + VC)) into
-    // the tile [y][z][VC] with asynchronous 16-byte copies (no register
+    // block b (x plane, VC velocity cells) into the tile [y][z][VC] with asynchronous 16-byte copies (no register
     // staging, few load instructions)
     auto stage = [&](long long b) {
         constexpr int Q = VC / 4, PIECES = N * N * Q;
-        const float *src = f + (b / nvb) * N * N * nvc + (b % nvb) * VC;
+        long long xp;
+        unsigned ch;
+        g.split(b, xp, ch);
+        const float *src = f + xp * N * N * nvc + (long long)ch * VC;
 #pragma unroll 4
         for (int e = t; e < PIECES; e += DriftYZ<N>::NT) {
             const int q = e % Q, yz = e / Q, y = yz / N, z = yz % N;
@@ -747,9 +751,14 @@ __global__ void __launch_bounds__(DriftYZ<N>::NT, 2) k_drift_yz(const float *__r
     };
     if ((long long)blockIdx.x < nblocks) stage(blockIdx.x);
     for (long long b = blockIdx.x; b < nblocks; b += gridDim.x) {
-        const long long v0 = (b % nvb) * VC;
-        const long long x0 = (b / nvb) * N * N;          // first spatial cell of the x plane
-        const long long v = v0 + 2 * vp;
+        long long xp;
+        unsigned ch;
+        int vy, vzc;
+        g.split(b, xp, ch);
+        g.velocity(ch, vy, vzc);
+        const long long x0 = xp * N * N;                 // first spatial cell of the x plane
+        const long long v = (long long)ch * VC + 2 * vp;
+        const int vz = vzc * VC + 2 * vp;
         float2 x[N];
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
@@ -758,7 +767,7 @@ __global__ void __launch_bounds__(DriftYZ<N>::NT, 2) k_drift_yz(const float *__r
             float *q = tile + r * YP + 2 * vp;
 #pragma unroll
             for (int j = 0; j < N; ++j) x[j] = *reinterpret_cast<const float2 *>(q + j * VC);
-            const LineCoef<float> ca = cz[(int)(v % nvz)], cb = cz[(int)((v + 1) % nvz)];
+            const LineCoef<float> ca = cz[vz], cb = cz[vz + 1];
             lost += drift_pair<N, PERIODIC>(x, ca, cb);
 #pragma unroll
             for (int j = 0; j < N; ++j) *reinterpret_cast<float2 *>(q + j * VC) = x[j];
@@ -774,7 +783,7 @@ __global__ void __launch_bounds__(DriftYZ<N>::NT, 2) k_drift_yz(const float *__r
         __syncthreads();
         if (b + gridDim.x < nblocks) stage(b + gridDim.x);
         {
-            const LineCoef<float> c = cy[(int)((v0 / nvz) % nvy)];
+            const LineCoef<float> c = cy[vy];
             lost += drift_pair<N, PERIODIC>(x, c, c);
             float *p = fo + (x0 + r) * nvc + v;
             const long long ys = (long long)N * nvc;
@@ -812,7 +821,8 @@ cudaError_t drift_yz_n(vp_ctx *c, const float *f, const LineCoef<float> *coef, f
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     long long grid = (long long)per_sm * vp_sm_count();
     if (grid > nblocks) grid = nblocks;
-    kern<<<(unsigned)grid, NT, smem, c->stream>>>(f, cz, cy, c->nvc, c->nv[1], c->nv[2], nblocks,
+    const YZBlocks g(c->nvc, c->nv[1], c->nv[2], DriftYZ<N>::VC);
+    kern<<<(unsigned)grid, NT, smem, c->stream>>>(f, cz, cy, c->nvc, g, nblocks,
                                                   &c->sc->lost, fo);
     return cudaGetLastError();
 }
