@@ -685,7 +685,9 @@ __global__ void __launch_bounds__(128) k_adjoint_rows(const float *__restrict__ 
 // back.  A cube with a whole-cell shift on any velocity axis is skipped:
 // all three of its sweeps go to the fix-up pass.  (A packed variant with two
 // rows or columns per lane needs 255 registers, leaves 8 warps per SM and
-// ran slower.)
+// ran slower.)  Bound by the latency of its phases at 16 warps per SM; each warp
+// fetches the rows of the warp that will take its place into L2: 32^6 3.75 -> 3.4-3.5
+// ms a pass (12 bytes per cell take 1.9 ms at 6.8 TB/s).
 template <int N>
 struct KickZY {
     static constexpr int P = N + 4, UPC = N * N / 32, WPC = 4;   // warps per CTA
@@ -698,7 +700,7 @@ __global__ void __launch_bounds__(128) k_kick_adjoint_zy(const float *__restrict
                                                         const LineCoef<float> *__restrict__ coef,
                                                         long long np, double *__restrict__ lam_g,
                                                         double scale_y, double scale_z,
-                                                        int *skipped)
+                                                        int *skipped, long long ahead)
 {
     constexpr int P = KickZY<N>::P, UPC = KickZY<N>::UPC;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -708,6 +710,11 @@ __global__ void __launch_bounds__(128) k_kick_adjoint_zy(const float *__restrict
     float *tc = tb + 32 * P;       // vz input rows (recomputed)
     const long long unit = (long long)blockIdx.x * KickZY<N>::WPC + warp;
     if (unit >= np * UPC) return;
+    // the rows of the warp that takes this one's place into L2
+    if (lane == 0 && unit + ahead < np * UPC) {
+        prefetch_l2(lam + (unit + ahead) * 32 * N, 32 * N * sizeof(float));
+        prefetch_l2(sb + (unit + ahead) * 32 * N, 32 * N * sizeof(float));
+    }
     const long long cell = unit / UPC;
     const LineCoef<float> cx = coef[cell * 3], cy = coef[cell * 3 + 1], cz = coef[cell * 3 + 2];
     if (((cx.code | cy.code | cz.code) >> 1) != 0) {
@@ -923,6 +930,13 @@ unsigned persistent_grid(K kernel, size_t smem, long long units)
     return (unsigned)(g < cap ? g : cap);
 }
 
+// warps of CTAs of 128 threads that fit on the SMs at once
+template <class K>
+long long resident_warps(K kernel, size_t smem)
+{
+    return 4LL * persistent_grid(kernel, smem, 1LL << 40);
+}
+
 // dynamic shared memory above the default 48 KB (static included) must be
 // allowed per kernel before its launch
 template <class K>
@@ -999,13 +1013,13 @@ cudaError_t launch_kick_adjoint3(vp_ctx *c, const void *sa, const void *sb, void
             return e;
         k_kick_adjoint_zy<32><<<grid, 32 * K::WPC, K::SMEM, c->stream>>>(
             (const float *)sb, (float *)lam, cf, c->np, lam_g, tau / c->dv[1], tau / c->dv[2],
-            c->adj_flag);
+            c->adj_flag, resident_warps(k_kick_adjoint_zy<32>, K::SMEM));
     } else {
         typedef KickZY<16> K;
         const unsigned grid = (unsigned)((c->np * K::UPC + K::WPC - 1) / K::WPC);
         k_kick_adjoint_zy<16><<<grid, 32 * K::WPC, K::SMEM, c->stream>>>(
             (const float *)sb, (float *)lam, cf, c->np, lam_g, tau / c->dv[1], tau / c->dv[2],
-            c->adj_flag);
+            c->adj_flag, resident_warps(k_kick_adjoint_zy<16>, K::SMEM));
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     return launch_adjoint_pairs(c, sa, lam, 3, coef, lam_g, tau / c->dv[0], nullptr, 1);
