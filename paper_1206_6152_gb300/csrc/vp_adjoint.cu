@@ -570,12 +570,11 @@ cudaError_t sweep_adjoint_t(vp_ctx *c, const T *fin, T *lam, int axis, const Lin
             fast = true;
         }
     }
-    // every other line of 3 to 64 cells: 2 to 4 times faster than the routine below at
-    // each size measured (vp_adjoint_lines.cu); shorter and longer ones stay there
-    if (!fast && vp_adjoint_lines_ok(c, axis)) {
-        if ((e = launch_adjoint_lines(c, fin, lam, axis, coef, lam_g, dalpha_scale)) != cudaSuccess) return e;
-        fast = true;
-    }
+    // every other line of 3 to 64 cells, shifted or not: 2 to 4 times faster than the
+    // routine below at each size measured (vp_adjoint_lines.cu); shorter and longer
+    // ones stay there
+    if (!fast && vp_adjoint_lines_ok(c, axis))
+        return launch_adjoint_lines(c, fin, lam, axis, coef, lam_g, dalpha_scale);
     if (fast) {
         // lines the register kernels skipped (whole-cell shifts), if any
         long long small = 4LL * vp_sm_count();

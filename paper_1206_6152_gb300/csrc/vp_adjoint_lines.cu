@@ -1,5 +1,5 @@
 // vp_adjoint_lines.cu -- adjoint sweeps of lines of any length from 3 to 64,
-// one line per thread (zero whole-cell shift): the transpose of one sweep with
+// one line per thread: the transpose of one sweep with
 // the limiter arms of vp_adjoint.cu's line_adjoint, each sum formed in its
 // order, so that the results are those of that routine bit for bit.
 //
@@ -10,7 +10,8 @@
 // j - 1); the input cotangent of a cell is complete one cell later:
 //   li_j = ((lp_{j-1} + l_j) + l0_j) + lm_{j+1},
 // for periodic lines with the wrapped terms where the routine adds them (lm_0
-// first in cell n - 1, lp_{n-1} last in cell 0).
+// first in cell n - 1, lp_{n-1} last in cell 0).  A whole-cell shift s only moves the
+// cotangent: cell j meets entries j + s and j + s + 1, wrapped or zero past the end.
 // Lines along x, y, z, vx and vy are copied element by element into the thread's
 // own slots (a warp copies neighbouring cells); vz rows go through a tile, rows
 // at odd pitch, with the CTA's contiguous rows copied in and out coalesced.
@@ -19,8 +20,8 @@
 // cycles per warp instruction): comparisons, doublings and selections of FP64 run
 // on the integer pipes, which leaves 13 FP64 instructions per cell, 17 with the
 // beta derivative.  Measured, one sweep: FP32 20 x 18 x 22 of 24 x 28 x 26 cells
-// (1.66 GB, 245 us at 6.8 TB/s) 360-400 us, vz 518 us, where the shared-memory
-// kernel of vp_adjoint.cu took 1140-1710 us; FP64 16^6 440 us (drifts) and 577-595 us
+// (1.66 GB, 245 us at 6.8 TB/s) 365-410 us, vz 534 us, where the shared-memory
+// kernel of vp_adjoint.cu took 1140-1710 us, shifted by whole cells or not; FP64 16^6 440 us (drifts) and 577-595 us
 // (kicks), where lines of all FP64 instructions in registers took 1120 us and, with
 // both directions in a warp, 2200 us; FP64 12 x 10 x 14 of 16 x 18 x 20 260-411 us,
 // shared memory 770-890 us.
@@ -150,7 +151,7 @@ struct AdjLines {
 template <typename T, int NMAX, bool PERIODIC, bool DB, bool ROWS>
 __global__ void __launch_bounds__(128) k_adjoint_lines(const T *__restrict__ fin, T *lam,
                                                       const LineCoef<T> *__restrict__ coef, AdjLines g,
-                                                      double *lam_g, double scale, int *skipped)
+                                                      double *lam_g, double scale)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red[32];
@@ -158,7 +159,7 @@ __global__ void __launch_bounds__(128) k_adjoint_lines(const T *__restrict__ fin
     const int t = threadIdx.x, NT = blockDim.x, n = g.n, P = n | 1;
     const bool kick = g.axis >= 3;
     const int u0 = (kick ? blockIdx.y : blockIdx.x) * NT, u = u0 + t;
-    bool active = u < g.inner;
+    const bool active = u < g.inner;
     long long off = 0;
     LineCoef<T> cf;
     cf.code = 0;
@@ -173,18 +174,15 @@ __global__ void __launch_bounds__(128) k_adjoint_lines(const T *__restrict__ fin
         off = ((o / g.od) * g.m1 + (o % g.od) * g.m2) * g.nvc + u;
         if (active) cf = coef[(u / g.va_stride) % g.va_n];
     }
-    if (active && (cf.code >> 1) != 0) {
-        atomicExch(skipped, 1);
-        active = false;
-    }
     const bool neg = cf.code & 1;
+    // entries of the output cotangent before the wrap (periodic) or the end
+    const int shift = PERIODIC ? (cf.code >> 1) % n : (cf.code >> 1 < n ? cf.code >> 1 : n), nb = n - shift;
     const long long st = neg ? -g.stride : g.stride, o0 = off + (neg ? (n - 1) * g.stride : 0);
     T x[NMAX + 1], fm1 = T(0);
     int cnt = 0;
     if constexpr (ROWS) {
-        // the CTA's rows (one cube: all skipped or none) through the tile, the
-        // state first, then the cotangent
-        if ((cf.code >> 1) != 0) return;
+        // the CTA's rows through the tile, the state first, then the cotangent (read at
+        // or past the cell that is written)
         cnt = (g.inner - u0 < NT ? g.inner - u0 : NT) * n;
         const T *src = fin + (off - (long long)t * n);
         const int dr = NT / n, dk = NT - dr * n;
@@ -216,7 +214,8 @@ __global__ void __launch_bounds__(128) k_adjoint_lines(const T *__restrict__ fin
             int arg;
             T lfinf, db;
             adjoint_line<T, NMAX, false, DB>(
-                x, n, T(0), cf, [&](int j) { return l[j * rs]; }, [&](int j, T v) { l[j * rs] = v; }, arg,
+                x, n, T(0), cf, [&](int j) { return j < nb ? l[(j + shift) * rs] : T(0); },
+                [&](int j, T v) { l[j * rs] = v; }, arg,
                 lfinf, db);
             l[arg * rs] += lfinf;
             da = neg ? -(double)db : (double)db;
@@ -246,7 +245,12 @@ __global__ void __launch_bounds__(128) k_adjoint_lines(const T *__restrict__ fin
         int arg;
         T lfinf, db;
         adjoint_line<T, NMAX, PERIODIC, DB>(
-            x, n, fm1, cf, [&](int j) { return l[j * NT]; }, [&](int j, T v) { lam[o0 + j * st] = v; }, arg,
+            x, n, fm1, cf,
+            [&](int j) {
+                if (!PERIODIC) return j < nb ? l[(j + shift) * NT] : T(0);
+                return l[(j < nb ? j + shift : j - nb) * NT];
+            },
+            [&](int j, T v) { lam[o0 + j * st] = v; }, arg,
             lfinf, db);
         lam[o0 + arg * st] += lfinf;
         da = neg ? -(double)db : (double)db;
@@ -267,7 +271,7 @@ cudaError_t go(vp_ctx *c, const T *fin, T *lam, const LineCoef<T> *coef, const A
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 72 * 1024);
         if (e != cudaSuccess) return e;
     }
-    kern<<<grid, NT, smem, c->stream>>>(fin, lam, coef, g, lam_g, scale, c->adj_flag);
+    kern<<<grid, NT, smem, c->stream>>>(fin, lam, coef, g, lam_g, scale);
     return cudaGetLastError();
 }
 
@@ -289,8 +293,6 @@ template <typename T>
 cudaError_t lines_t(vp_ctx *c, const T *fin, T *lam, int axis, const LineCoef<T> *coef, double *lam_g,
                     double scale)
 {
-    cudaError_t e = cudaMemsetAsync(c->adj_flag, 0, sizeof(int), c->stream);
-    if (e != cudaSuccess) return e;
     AdjLines g{};
     g.axis = axis;
     g.nvc = c->nvc;
@@ -330,7 +332,7 @@ int vp_adjoint_lines_ok(const vp_ctx *c, int axis)
     const int n = axis < 3 ? c->n[axis] : c->nv[axis - 3];
     // (the grid's y dimension: outer indices for the position axes, chunks of 128
     // lines for the velocity axes; the lines of one outer index count in an int)
-    return c->adj_flag && n >= 3 && n <= 64 && c->nvc <= (1LL << 30) &&
+    return n >= 3 && n <= 64 && c->nvc <= (1LL << 30) &&
            (axis < 3 ? c->np / n <= 65535 : c->nvc / n <= 65535LL * 128);
 }
 

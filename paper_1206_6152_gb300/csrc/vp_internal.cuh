@@ -213,8 +213,8 @@ cudaError_t launch_field_adjoint(vp_ctx *c, const double *lam_g, void *lam_f, bo
 // FP32 packed register-line adjoint sweeps (line lengths 16/32/48, zero
 // whole-cell shift; skipped lines set c->adj_flag)
 int vp_adjoint_pairs_ok(const vp_ctx *c, int axis);
-// one adjoint sweep of lines of any length from 3 to 64, zero shift (skipped
-// lines set c->adj_flag); lam_g (all three axes) for the velocity axes, or null
+// one adjoint sweep of lines of any length from 3 to 64 (any shift); lam_g (all
+// three axes) for the velocity axes, or null
 int vp_adjoint_lines_ok(const vp_ctx *c, int axis);
 cudaError_t launch_adjoint_lines(vp_ctx *c, const void *fin, void *lam, int axis, const void *coef,
                                  double *lam_g, double scale);
