@@ -531,19 +531,15 @@ __device__ __forceinline__ long long unit_to_v(long long L, const DriftGeom &g)
 // pair) visits, live in shared memory (slot j of pair q at 128 j + q, or at q ^ 8 for odd
 // j of the lanes' form: conflict-free); the rows of the CTA's next lines are fetched into L2.
 // What bounds it: HBM; with the density, lines of 48 and 64 in pairs (255 registers, 8
-// warps per SM) were bound by latency, so these take one line per thread (16 warps;
+// warps per SM) were bound by latency, so these go one line per thread (SINGLE: 16 warps;
 // the lanes of a pair exchange cells so that each sum is formed in the pairs' order).
 // Measured, x drift: 64 x 32^2 of 32^3 cells (2.5 ms at 6.8 TB/s) 3.90 -> 3.46 ms, 64 x 16^2
-// 1.40 -> 0.95 ms, 48 x 16^2 of 48^3 2.16 -> 2.02 ms; the fetch alone 32^6 1.48 -> 1.45 ms,
+// 1.40 -> 0.95 ms, 48 x 16^2 of 48^3 2.16 -> 2.02 ms (48^6 stays in pairs: 15.8 -> 15.7 with the
+// fetch, single lines 16.4); the fetch alone 32^6 1.48 -> 1.45 ms,
 // 16^3 of 32^3 234 -> 222 us.  Without the density pairs stay: single lines of 48 were
 // slower (y, z drift of 16 x 48^2 of 48^3 5.1 -> 5.3 ms), as were lines of 64 (804 -> 873 us).
-template <int N, bool RHO>
-constexpr bool drift_single = RHO && N > 32;      // one line per thread, not a pair
-template <int N, bool RHO>
-constexpr int drift_threads = drift_single<N, RHO> ? 256 : 128;
-
-template <int N, bool PERIODIC, bool RHO>
-__global__ void __launch_bounds__(drift_threads<N, RHO>, N <= 32 ? 4 : (RHO ? 2 : 1)) k_drift_fast(const float *__restrict__ f,
+template <int N, bool PERIODIC, bool SINGLE, bool RHO>
+__global__ void __launch_bounds__(SINGLE ? 256 : 128, N <= 32 ? 4 : (SINGLE ? 2 : 1)) k_drift_fast(const float *__restrict__ f,
                                                                const LineCoef<float> *__restrict__ coef,
                                                                DriftGeom g, double *__restrict__ rho_part,
                                                                double *lost_out, float *__restrict__ fo)
@@ -569,7 +565,7 @@ __global__ void __launch_bounds__(drift_threads<N, RHO>, N <= 32 ? 4 : (RHO ? 2 
         }
     };
     float lost = 0.f;
-    if constexpr (!drift_single<N, RHO>) {
+    if constexpr (!SINGLE) {
         sacc += t;
         if constexpr (RHO) {
 #pragma unroll
@@ -916,13 +912,21 @@ cudaError_t drift_fast_n(vp_ctx *c, float *f, int axis, const LineCoef<float> *c
     double *lost = &c->sc->lost;
     if (rho_part) {
         constexpr size_t racc = (size_t)N * 128 * sizeof(Acc<float>);   // density sums
-        auto kern = c->periodic_space ? k_drift_fast<N, true, true> : k_drift_fast<N, false, true>;
+        // lines of more than 32 cells singly, but those of 48 in pairs where a CTA has more
+        // than a hundred turns (48^6, 216 turns: 15.7 ms against 16.4; 48 x 32^2 of 32^3, 43
+        // turns: 2.51 against 2.36)
+        constexpr bool LONG = N > 32;
+        const bool single = LONG && (N != 48 || g.per_part <= 100 * 128);
+        auto kern = c->periodic_space ? k_drift_fast<N, true, LONG, true> : k_drift_fast<N, false, LONG, true>;
+        if constexpr (N == 48) {
+            if (!single) kern = c->periodic_space ? k_drift_fast<N, true, false, true> : k_drift_fast<N, false, false, true>;
+        }
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)racc);
         if (e != cudaSuccess) return e;
-        kern<<<grid, drift_threads<N, true>, racc, c->stream>>>(f, coef, g, rho_part, lost, o);
+        kern<<<grid, single ? 256 : 128, racc, c->stream>>>(f, coef, g, rho_part, lost, o);
     } else {
-        auto kern = c->periodic_space ? k_drift_fast<N, true, false> : k_drift_fast<N, false, false>;
-        kern<<<grid, drift_threads<N, false>, 0, c->stream>>>(f, coef, g, rho_part, lost, o);
+        auto kern = c->periodic_space ? k_drift_fast<N, true, false, false> : k_drift_fast<N, false, false, false>;
+        kern<<<grid, 128, 0, c->stream>>>(f, coef, g, rho_part, lost, o);
     }
     return cudaGetLastError();
 }
