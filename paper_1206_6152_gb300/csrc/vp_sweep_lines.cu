@@ -51,7 +51,8 @@ namespace {
 // FP32 sums are kept and merged as double-floats on the FP32 pipe, one FP64
 // addition per warp at the end.  FP64: merging a CTA's threads takes about 50
 // FP64 instructions a warp, so it is done once per CTA of a grid that just
-// fills the SMs, not once per line.
+// fills the SMs, not once per line.  Both merges shuffle whole warps: a CTA has a
+// multiple of 32 threads (a lane that does not exist has no defined value).
 template <typename T>
 struct Lost;
 template <>
@@ -345,10 +346,12 @@ __global__ void __launch_bounds__(512) k_kick_blocks(const float *src, float *ds
 // from global memory (coalesced along vz), through the tile (row pitch N + 4: 16
 // bytes aligned, rows free of bank conflicts) to vz rows read and written 16
 // bytes at a time, and out of it with coalesced 16-byte stores; the CTA's next
-// planes are fetched into L2 meanwhile.
+// planes are fetched into L2 meanwhile.  CTAs of whole warps, as add_lost's merge
+// needs: two planes of 40 or 56 lines leave 16 threads that take no line and join the
+// barriers and the merge only.
 template <int N>
 struct Planes {
-    static constexpr int G = 2, NT = G * N, P = N + 4;
+    static constexpr int G = 2, NT = (G * N + 31) / 32 * 32, P = N + 4;
     static constexpr size_t SMEM = (size_t)G * N * P * sizeof(float);
 };
 
@@ -367,6 +370,7 @@ __global__ void __launch_bounds__(Planes<N>::NT) k_kick_planes(const float *src,
                                                                double *lost_out)
 {
     typedef Planes<N> B;
+    static_assert(B::NT % 32 == 0, "add_lost merges whole warps");
     constexpr int P = B::P, NN = N * N, Q = N / 4;
     extern __shared__ __align__(16) float tile[];
     const int t = threadIdx.x, g = t / N, m = t % N, per = (nx + B::G - 1) / B::G;
