@@ -141,7 +141,61 @@ __device__ __forceinline__ T clamp_line(const T (&x)[NMAX + 1], int n, T fm1, T 
     return phm;
 }
 
-// the same for FP32 lines of N cells known at compile time, in array order and
+// the update of the outflow line x moved on by s whole cells as well (0 <= s <= n),
+// in the arithmetic and the order of sums of kick_line_shifted (vp_fast_line.cuh): cell
+// j and the flux before it go to position j + s, cells that would pass the end are
+// lost, positions below s are empty (the caller's to write).  put(v) takes the new
+// values of positions s, s + 1, ... in turn.  Returns what leaves.  Only the fluxes of
+// cells that stay are computed, so a sweep by several cells takes about as long as one
+// by a part of one; line by line in place in global memory, two reads per cell and no
+// more than one under way, the vz sweep of 8^3 cubes of 64^3 took 1440 us (now 190-270).
+template <typename T, int NMAX, class P>
+__device__ __forceinline__ T clamp_line_shifted(const T (&x)[NMAX + 1], int n, int s, T c0, T c1, T c2,
+                                                P put)
+{
+    const T finf = clamp_line_max<T, NMAX, 1>(x, n);
+    T dm = x[0], phm = T(0), lost = T(0);
+    const int stay = n - s;
+#pragma unroll
+    for (int j = 0; j < NMAX; ++j) {
+        if (j >= n) break;
+        if (j < stay) {
+            const T dp = x[j + 1] - x[j];
+            const T ph = clamp_flux(dm, x[j], dp, finf, c0, c1, c2);
+            put((x[j] - ph) + phm);
+            phm = ph;
+            dm = dp;
+        } else {
+            lost += x[j];
+        }
+    }
+    return lost + phm;
+}
+
+// The same from p (step sp) to w (step sw; p may be w), both at the upwind end, shared or
+// global memory.  A call: inlined beside the sub-cell code of lines in global memory, of
+// planes and of blocks of lines above 32 cells it took registers and instruction fetches
+// that made the sub-cell sweeps 2 to 5 % slower.
+template <typename T, int NMAX>
+__device__ __noinline__ T shifted_line(const T *p, int sp, T *w, int sw, int n, const LineCoef<T> cf)
+{
+    const int s = cf.code >> 1 < n ? cf.code >> 1 : n;
+    T x[NMAX + 1];
+    load_line<T, NMAX, false, 1>(x, n, [&]() {
+        const T v = *p;
+        p += sp;
+        asm volatile("" : "+l"(p));
+        return v;
+    });
+    for (int j = 0; j < s; ++j, w += sw) *w = T(0);
+    return clamp_line_shifted<T, NMAX>(x, n, s, cf.c0, cf.c1, cf.c2, [&](T v) {
+        *w = v;
+        w += sw;
+        asm volatile("" : "+l"(w));
+    });
+}
+
+// clamp_line for FP32 lines of N cells known at compile time, in array order and
 // in place (outflow)
 template <int N, bool NEG>
 __device__ __forceinline__ float clamp_exact(float (&x)[N], float finf, float c0, float c1, float c2)

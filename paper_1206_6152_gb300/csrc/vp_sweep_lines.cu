@@ -1,8 +1,7 @@
 // vp_sweep_lines.cu -- sweeps along lines of any length up to 64 cells, one
-// line per thread in registers (zero whole-cell shift; vp_clamp_line.cuh).
-// These serve every grid whose lengths have no kernel of their own; the
-// shared-memory kernels of vp_sweep.cu remain for longer lines and for shifts
-// of one cell or more.
+// line per thread in registers (vp_clamp_line.cuh).  These serve every grid whose
+// lengths have no kernel of their own; the shared-memory kernels of vp_sweep.cu
+// remain for longer lines and for drifts by one cell or more.
 //
 //  * k_drift_lines: lines along a spatial axis straight from global memory to
 //    registers and back (a warp reads 32 neighbouring velocity cells per
@@ -19,10 +18,11 @@
 //    ran both directions' code in every warp (16^6: 0.59 -> 0.25 ms).
 //  * k_kick_lines: one velocity sweep of every cube, the same way (vx and vy
 //    lines: a warp reads neighbouring cells; vz: each thread its own row, whose
-//    32-byte sectors it uses up over consecutive loads).  A line with a
-//    whole-cell shift takes the generic in-place routine.  FP64 cubes go
-//    through it one launch per sweep: at 16 bytes per cell the sweep is bound by
-//    the FP64 pipe alone.
+//    32-byte sectors it uses up over consecutive loads).  FP64 cubes go through it
+//    one launch per sweep: at 16 bytes per cell the sweep is bound by the FP64 pipe
+//    alone.  A line that moves by whole cells is held in registers as well
+//    (shifted_line): in place in global memory, sweeps of 24 x 28 x 26 cubes by 1.5
+//    cells took 420 us where one by 0.4 of a cell takes 250, now 285.
 //  * k_kick_blocks: FP32 cubes in blocks of vx planes in shared memory: whole
 //    cubes, all sweeps of a kick in one pass, where they fit (220 KB); larger
 //    ones as one pass per vx sweep (k_kick_lines) and one per run of vy and vz
@@ -151,8 +151,17 @@ __global__ void __launch_bounds__(128) k_drift_lines(const T *f, const LineCoef<
     if (!PERIODIC) add_lost(lost, lost_out);
 }
 
+// CTAs per SM that the sub-cell code alone leaves room for (the function for lines that
+// move by whole cells would take registers of its own beyond that)
 template <typename T, int NMAX>
-__global__ void __launch_bounds__(128) k_kick_lines(const T *src, T *dst,
+constexpr int kick_lines_ctas()
+{
+    if (sizeof(T) == 8) return NMAX <= 16 ? 7 : (NMAX <= 32 ? 4 : 3);
+    return NMAX <= 16 ? 10 : (NMAX <= 32 ? 8 : (NMAX <= 48 ? 6 : 5));
+}
+
+template <typename T, int NMAX>
+__global__ void __launch_bounds__(128, kick_lines_ctas<T, NMAX>()) k_kick_lines(const T *src, T *dst,
                                                    const LineCoef<T> *__restrict__ coef, int va,
                                                    int nx, int ny, int nz, long long np,
                                                    double *lost_out)
@@ -171,16 +180,14 @@ __global__ void __launch_bounds__(128) k_kick_lines(const T *src, T *dst,
         else { base = u * nz; step = 1; }
         const LineCoef<T> cf = coef[cell * 3 + va];
         const long long off = cell * nvc + base;
-        if ((cf.code >> 1) != 0) {
-            if (src != dst)
-                for (int j = 0; j < n; ++j) dst[off + (long long)j * step] = src[off + (long long)j * step];
-            lost.add(kick_line_shifted(dst + off, step, n, cf));
-            continue;
-        }
         const bool neg = cf.code & 1;
         const int st = neg ? -step : step;
         const T *p = src + off + (neg ? (n - 1) * step : 0);
         T *w = dst + off + (neg ? (n - 1) * step : 0);
+        if ((cf.code >> 1) != 0) {
+            lost.add(shifted_line<T, NMAX>(p, st, w, st, n, cf));
+            continue;
+        }
         T x[NMAX + 1];
         load_line<T, NMAX, false, 1>(x, n, [&]() { return next(p, st); });
         lost.add(clamp_line<T, NMAX, false, 1>(x, n, T(0), T(0), cf.c0, cf.c1, cf.c2, [&](int, T v) {
@@ -231,8 +238,9 @@ __device__ __forceinline__ void each_element(int count, int nz, F f)
 // one sweep of the block's lines along va, from src (IN) or the tile, into dst
 // (OUT) or the tile; which one it is is known at compile time, so that the tile
 // is addressed as shared memory (with one generic pointer for both a cell took
-// 35 instructions and the 24 x 28 x 26 kick 1.14 ms)
-template <int NMAX, bool IN, bool OUT>
+// 35 instructions and the 24 x 28 x 26 kick 1.14 ms).  SHIFT: lines that move by
+// whole cells, in the tile
+template <int NMAX, bool IN, bool OUT, bool SHIFT = false>
 __device__ __forceinline__ void sweep_lines(const Block &B, int va, const float *src, float *dst, float *tile,
                             const LineCoef<float> &c, Lost<float> &lost)
 {
@@ -242,6 +250,10 @@ __device__ __forceinline__ void sweep_lines(const Block &B, int va, const float 
     for (int u = threadIdx.x; u < L; u += blockDim.x) {
         const int a = B.first(va, u, P) + (neg ? (1 - n) * sp : 0);
         const int g = IN || OUT ? B.first(va, u, nz) + (neg ? (1 - n) * sg : 0) : 0;
+        if constexpr (SHIFT && NMAX > 32) {
+            lost.add(shifted_line<float, NMAX>(tile + a, sp, tile + a, sp, n, c));
+            continue;
+        }
         float x[NMAX + 1];
         if constexpr (IN) {
             const float *p = src + g;
@@ -254,6 +266,17 @@ __device__ __forceinline__ void sweep_lines(const Block &B, int va, const float 
                 asm volatile("" : "+r"(q));
                 return v;
             });
+        }
+        if constexpr (SHIFT) {
+            const int s = c.code >> 1 < n ? c.code >> 1 : n;
+            for (int j = 0; j < s; ++j) tile[a + j * sp] = 0.f;
+            int q = 4 * (a + s * sp);
+            lost.add(clamp_line_shifted<float, NMAX>(x, n, s, c.c0, c.c1, c.c2, [&](float v) {
+                *reinterpret_cast<float *>(reinterpret_cast<char *>(tile) + q) = v;
+                q += 4 * sp;
+                asm volatile("" : "+r"(q));
+            }));
+            continue;
         }
         float *w = dst + g;
         int r = 4 * a;
@@ -281,7 +304,7 @@ __device__ __forceinline__ void sweep_block(const Block &B, const float *src, fl
                                             const LineCoef<float> *cf, int nsweeps, int first_axis,
                                             Lost<float> &lost)
 {
-    const int nz = B.nz, P = nz | 1, rows = B.g * B.ny;
+    const int nz = B.nz, rows = B.g * B.ny;
     auto whole = [&](int sw) { return (cf[sw].code >> 1) != 0; };
     const bool in = first_axis < 2 && !whole(0);
     if (!in) {
@@ -294,9 +317,7 @@ __device__ __forceinline__ void sweep_block(const Block &B, const float *src, fl
         const LineCoef<float> c = cf[sw];
         out = sw == nsweeps - 1 && va < 2 && !whole(sw);
         if (whole(sw)) {
-            const int n = B.len(va), st = B.step(va, P);
-            for (int u = threadIdx.x; u < B.lines(va); u += blockDim.x)
-                lost.add(kick_line_shifted(tile + B.first(va, u, P), st, n, c));
+            sweep_lines<NMAX, false, false, true>(B, va, src, dst, tile, c, lost);
         } else if (sw == 0 && in) {
             if (out) sweep_lines<NMAX, true, true>(B, va, src, dst, tile, c, lost);
             else sweep_lines<NMAX, true, false>(B, va, src, dst, tile, c, lost);
@@ -353,6 +374,7 @@ template <int N>
 struct Planes {
     static constexpr int G = 2, NT = (G * N + 31) / 32 * 32, P = N + 4;
     static constexpr size_t SMEM = (size_t)G * N * P * sizeof(float);
+    static constexpr int CTAS = N <= 40 ? 9 : (N <= 48 ? 8 : (N <= 56 ? 6 : 4));   // as kick_lines_ctas
 };
 
 template <int N>
@@ -364,7 +386,7 @@ __device__ __forceinline__ float sweep_exact(float (&x)[N], const LineCoef<float
 }
 
 template <int N>
-__global__ void __launch_bounds__(Planes<N>::NT) k_kick_planes(const float *src, float *dst,
+__global__ void __launch_bounds__(Planes<N>::NT, Planes<N>::CTAS) k_kick_planes(const float *src, float *dst,
                                                                const LineCoef<float> *__restrict__ coef,
                                                                int do1, int do2, int nx, long long np,
                                                                double *lost_out)
@@ -382,25 +404,23 @@ __global__ void __launch_bounds__(Planes<N>::NT) k_kick_planes(const float *src,
         const long long off = (cell * nx + i0) * NN, un = u + gridDim.x;
         const float *s = src + off;
         float *d = dst + off;
-        if ((do1 && (c1.code >> 1) != 0) || (do2 && (c2.code >> 1) != 0)) {
-            // a whole-cell shift: line by line in dst
-            if (src != dst)
-                for (int e = t; e < planes * NN; e += B::NT) d[e] = s[e];
-            __syncthreads();
-            if (do1 && g < planes) lost.add(kick_line_shifted(d + g * NN + m, N, N, c1));
-            __syncthreads();
-            if (do2 && g < planes) lost.add(kick_line_shifted(d + g * NN + m * N, 1, N, c2));
-            __syncthreads();
-            continue;
-        }
+        // (uniform over the CTA) a sweep that moves by whole cells: lines in upwind order
+        const bool shifted = (do1 && (c1.code >> 1) != 0) || (do2 && (c2.code >> 1) != 0);
         float x[N];
-        if (g < planes) {
+        if (g < planes && !shifted) {
             // vy line (plane g, vz = m)
 #pragma unroll
             for (int j = 0; j < N; ++j) x[j] = s[g * NN + j * N + m];
             if (do1) lost.add(sweep_exact<N>(x, c1));
 #pragma unroll
             for (int j = 0; j < N; ++j) tile[(g * N + j) * P + m] = x[j];
+        } else if (g < planes) {
+            const int j0 = c1.code & 1 ? N - 1 : 0, d1 = c1.code & 1 ? -1 : 1;
+            const float *p = s + (g * N + j0) * N + m;
+            float *q = tile + (g * N + j0) * P + m;
+            if (do1) lost.add(shifted_line<float, N>(p, d1 * N, q, d1 * P, N, c1));
+            else
+                for (int j = 0; j < N; ++j) q[j * d1 * P] = p[j * d1 * N];
         }
         if (t == 0 && un < np * per) {
             const long long cn = un / per;
@@ -410,7 +430,7 @@ __global__ void __launch_bounds__(Planes<N>::NT) k_kick_planes(const float *src,
                          : "memory");
         }
         __syncthreads();
-        if (do2 && g < planes) {
+        if (do2 && g < planes && !shifted) {
             // vz row (plane g, vy = m)
             float4 *r = reinterpret_cast<float4 *>(tile + (g * N + m) * P);
 #pragma unroll
@@ -422,6 +442,10 @@ __global__ void __launch_bounds__(Planes<N>::NT) k_kick_planes(const float *src,
 #pragma unroll
             for (int q = 0; q < Q; ++q)
                 r[q] = make_float4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]);
+        } else if (do2 && g < planes) {
+            const int d2 = c2.code & 1 ? -1 : 1;
+            float *r = tile + (g * N + m) * P + (c2.code & 1 ? N - 1 : 0);
+            lost.add(shifted_line<float, N>(r, d2, r, d2, N, c2));
         }
         __syncthreads();
 #pragma unroll 4

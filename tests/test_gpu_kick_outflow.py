@@ -1,7 +1,8 @@
 """The mass that leaves through the velocity faces (M_out) in FP32 kicks of cubes
 whose vx planes have a kernel of a compile-time edge, against the FP64 oracle:
 edges whose pairs of planes are (48, 64) and are not (40, 56) a whole number of
-warps of lines, a last block of one plane, sweeps below a cell and of more."""
+warps of lines, a last block of one plane, sweeps below a cell, of more, and past
+the whole line."""
 import numpy as np
 import pytest
 
@@ -16,7 +17,7 @@ DEV = "cuda:0"
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("cells", [0.7, 1.6])
+@pytest.mark.parametrize("cells", [0.7, 1.6, 3.3, 70.0])
 @pytest.mark.parametrize("nv", [(37, 40, 40), (25, 48, 48), (19, 56, 56), (15, 64, 64)])
 def test_outflow_of_plane_kicks_matches_oracle(nv, cells):
     from paper_1206_6152_gb300 import build as B
