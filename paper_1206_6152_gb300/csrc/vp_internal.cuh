@@ -187,7 +187,7 @@ cudaError_t launch_kick_lines(vp_ctx *c, const void *f, const void *ca, const vo
 // (vp_sweep_cells.cu)
 int vp_drift_cells_ok(const vp_ctx *c, int axis);
 cudaError_t launch_drift_cells(vp_ctx *c, const void *f, int axis, const void *coef, void *fo);
-int vp_kick_cells_ok(const vp_ctx *c);
+int vp_kick_cells_ok(const vp_ctx *c, int nsweeps, int first_axis);
 cudaError_t launch_kick_cells(vp_ctx *c, const void *f, const void *ca, const void *cb, int nsweeps,
                               int first_axis, void *fo);
 // one sweep from src into dst (dst != src), used by the adjoint's replay;

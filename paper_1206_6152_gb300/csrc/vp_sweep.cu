@@ -666,7 +666,7 @@ cudaError_t launch_kick(vp_ctx *c, void *f, const void *coef_a, const void *coef
 {
     if (vp_kick_fast_ok(c)) return launch_kick_fast(c, f, coef_a, coef_b, nsweeps, first_axis);
     if (vp_kick_big_ok(c)) return launch_kick_big(c, f, coef_a, coef_b, nsweeps, first_axis);
-    if (vp_kick_cells_ok(c)) return launch_kick_cells(c, f, coef_a, coef_b, nsweeps, first_axis, f);
+    if (vp_kick_cells_ok(c, nsweeps, first_axis)) return launch_kick_cells(c, f, coef_a, coef_b, nsweeps, first_axis, f);
     if (vp_kick_lines_ok(c)) return launch_kick_lines(c, f, coef_a, coef_b, nsweeps, first_axis, f);
     if (c->isdouble)
         return launch_kick_dispatch<double>(c, (double *)f, (const LineCoef<double> *)coef_a,
@@ -683,7 +683,7 @@ cudaError_t launch_sweep_into(vp_ctx *c, const void *src, void *dst, int axis, c
         return launch_kick_fast(c, const_cast<void *>(src), coef, nullptr, 1, axis - 3, dst);
     if (axis >= 3 && vp_kick_big_ok(c))
         return launch_kick_big(c, const_cast<void *>(src), coef, nullptr, 1, axis - 3, dst);
-    if (axis >= 3 && vp_kick_cells_ok(c))
+    if (axis >= 3 && vp_kick_cells_ok(c, 1, axis - 3))
         return launch_kick_cells(c, src, coef, nullptr, 1, axis - 3, dst);
     if (axis >= 3 && vp_kick_lines_ok(c))
         return launch_kick_lines(c, src, coef, nullptr, 1, axis - 3, dst);

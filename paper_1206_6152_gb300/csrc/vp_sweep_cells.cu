@@ -229,18 +229,19 @@ cudaError_t launch_drift_cells(vp_ctx *c, const void *f, int axis, const void *c
 
 // cubes whose two buffers and line maxima fit in 96 KB, where a cube's CTA (its
 // cells over 128 lanes, a round of cubes for every SM) is cheaper than one
-// thread per line: 128 cubes of 128 cells are by far, 4^3 cubes of 16^3 are not
-// (three steps 635 us against 362 us)
-int vp_kick_cells_ok(const vp_ctx *c)
+// thread per line along the axes swept: 128 cubes of 128 cells are by far, 4^3 cubes
+// of 16^3 are not (three steps 635 us against 362 us), and a single vy sweep of 6^3
+// cubes of 64 x 4 x 4 is not either, though the kick is
+int vp_kick_cells_ok(const vp_ctx *c, int nsweeps, int first_axis)
 {
     int nmin = c->nv[0];
-    double lines = 0.0;
-    for (int a = 0; a < 3; ++a) {
+    for (int a = 1; a < 3; ++a)
         if (c->nv[a] < nmin) nmin = c->nv[a];
-        lines += lines_cost(c, c->nv[a]);
-    }
+    const int axes = nsweeps < 3 ? nsweeps : 3;
+    double lines = 0.0;
+    for (int k = 0; k < axes; ++k) lines += lines_cost(c, c->nv[(first_axis + k) % 3]);
     const long long sms = vp_sm_count();
-    const double cells = 3 * 9.0 * (double)((c->np + sms - 1) / sms) * (double)((c->nvc + 127) / 128);
+    const double cells = axes * 9.0 * (double)((c->np + sms - 1) / sms) * (double)((c->nvc + 127) / 128);
     return c->isdouble && cells < lines && (2 * c->nvc + c->nvc / nmin) * sizeof(double) <= 96 * 1024;
 }
 
