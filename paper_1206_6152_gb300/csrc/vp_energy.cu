@@ -10,8 +10,10 @@
 //    and TwoProd with vx^2 in three floats: 19 FP32 instructions per cell, close
 //    to what HBM takes) and added to FP64 totals once per column.
 //    32^3 x 32^3 cells: 39.8 ms with two FP64 compensated sums per cell, 0.81 ms
-//    now.  A cell whose sum is so small or large that the double-floats' low
-//    parts could underflow or the products overflow is summed in FP64 instead.
+//    now.  The weights are taken in units of a power of two near the largest |v|^2, so
+//    that no unit of velocity brings the products near the ends of the FP32 range.  A
+//    cell whose sums are so small or large that low parts could underflow or a sum
+//    overflow is summed in FP64 instead.
 //  * k_energy_sums: the compensated sums over the spatial cells, of these and of
 //    rho phi (or the density misfit), by as many CTAs as pay; the last to arrive
 //    adds the CTAs' sums in order.
@@ -132,13 +134,13 @@ __device__ void cell_sums_f64(const T *q, int nx, int ny, int nz, const double *
 
 // G threads of a CTA of 256 per cell: 32 where there are cells enough to fill
 // the SMs with one warp each, else the whole CTA.  v: the cell centres along vx,
-// vy, vz, one after the other.
+// vy, vz, one after the other; v2exp: exponent of the largest |v|^2.
 template <typename T, int VEC, int G>
 __global__ void __launch_bounds__(256) k_energy_partials(const T *__restrict__ f, long long np, int nx,
                                                         int ny, int nz, const double *vcx,
                                                         const double *vcy, const double *vcz,
-                                                        double *__restrict__ partials, double dvol,
-                                                        double *__restrict__ rho)
+                                                        int v2exp, double *__restrict__ partials,
+                                                        double dvol, double *__restrict__ rho)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red[2][8];
@@ -148,7 +150,7 @@ __global__ void __launch_bounds__(256) k_energy_partials(const T *__restrict__ f
     for (int e = t; e < nt; e += 256) {
         const double u = e < nx ? vcx[e] : (e < nx + ny ? vcy[e - nx] : vcz[e - nx - ny]);
         v[e] = u;
-        v2[e] = split(u * u);
+        v2[e] = split(scalbn(u * u, -v2exp));
     }
     __syncthreads();
     const int nvc = nx * ny * nz, g = t % G;
@@ -172,8 +174,11 @@ __global__ void __launch_bounds__(256) k_energy_partials(const T *__restrict__ f
         if constexpr (sizeof(T) == 4) {
             cell_sums<VEC>(q, nx, ny, nz, v2, g, G, M, Q);
             merge(M, Q);
-            const double a = fabs(M);
-            if (!(a == 0.0 || (a > 1e-20 && a < 1e30))) {
+            // (low parts below 2^-126 are flushed: at most a few times that per cell of f,
+            // and as much of each weight)
+            const double a = fabs(M), b = fabs(Q), lo = nvc * 0x1p-70;
+            Q = scalbn(Q, v2exp);
+            if (!((a == 0.0 && b == 0.0) || (a > lo && a < 1e30 && b > lo && b > a * 0x1p-70 && b < 1e30))) {
                 cell_sums_f64(q, nx, ny, nz, v, g, G, M, Q);
                 merge(M, Q);
             }
@@ -246,8 +251,14 @@ cudaError_t partials_t(vp_ctx *c, const T *f, double *partials, double *rho)
     auto kern = warp ? k_energy_partials<T, VEC, 32> : k_energy_partials<T, VEC, 256>;
     long long grid = warp ? (c->np + 7) / 8 : c->np;
     if (grid > 8LL * vp_sm_count()) grid = 8LL * vp_sm_count();
+    double v2 = 0.0;
+    for (int a = 0; a < 3; ++a) {
+        const double v = fmax(fabs(c->cfg.vlo[a] + 0.5 * c->dv[a]), fabs(c->cfg.vhi[a] - 0.5 * c->dv[a]));
+        v2 += v * v;
+    }
+    const int v2exp = v2 > 0.0 && isfinite(v2) ? ilogb(v2) : 0;
     kern<<<(unsigned)grid, 256, smem, c->stream>>>(f, c->np, c->nv[0], c->nv[1], c->nv[2], c->vc[0],
-                                                   c->vc[1], c->vc[2], partials, c->dvol_v, rho);
+                                                   c->vc[1], c->vc[2], v2exp, partials, c->dvol_v, rho);
     return cudaGetLastError();
 }
 
