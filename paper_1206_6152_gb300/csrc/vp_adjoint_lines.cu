@@ -47,6 +47,13 @@ __device__ __forceinline__ bool less(double a, double b)
 {
     return dkey(a) < dkey(b) && !nan64(a) && !nan64(b);
 }
+// below 0 (-0 is not)
+__device__ __forceinline__ bool negative(float a) { return a < 0.f; }
+__device__ __forceinline__ bool negative(double a)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(a);
+    return b > 0x8000000000000000ULL && b <= 0xfff0000000000000ULL;
+}
 __device__ __forceinline__ bool nonzero(float a) { return a != 0.f; }
 __device__ __forceinline__ bool nonzero(double a) { return __double_as_longlong(a) << 1 != 0; }
 __device__ __forceinline__ float fused(float a, float b, float c) { return __fmaf_rn(a, b, c); }
@@ -101,8 +108,8 @@ __device__ __forceinline__ void adjoint_line(const T (&x)[NMAX + 1], int n, T fm
         const T l2 = j + 1 < n ? lo(j + 1) : (PERIODIC ? l0first : T(0));
         const T mu = l2 - l1, f0 = x[j], dp = x[j + 1] - f0;
         const T up = twice(f0), gap = twice(finf - f0), nup = negate(up), ngap = negate(gap);
-        const bool dpos = less(T(0), dp), dneg = less(dp, T(0));
-        const bool mpos = less(T(0), dm), mneg = less(dm, T(0));
+        const bool dpos = less(T(0), dp), dneg = negative(dp);
+        const bool mpos = less(T(0), dm), mneg = negative(dm);
         const bool pu = dpos && less(up, dp), pl = dneg && less(dp, ngap);
         const bool mh = mpos && less(gap, dm), ml = mneg && less(dm, nup);
         const bool plim = pu || pl, mlim = mh || ml;
