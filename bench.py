@@ -393,6 +393,17 @@ def _ncu_launches(csv_path):
     return [launches[i] for i in sorted(launches)]
 
 
+def _drift_with_density(name):
+    """True for the x drift with the fused density: the last template argument of
+    k_drift_fast<N, PERIODIC, SINGLE, RHO> in a kernel name, which ncu prints as 1,
+    (bool)1 or true."""
+    arg = name.split("k_drift_fast<")[1].split(">(")[0].rstrip("> ").split(",")[-1]
+    arg = arg.strip().replace("(bool)", "")
+    if arg not in ("0", "1", "false", "true"):
+        raise ValueError(f"unknown form of kernel name: {name}")
+    return arg in ("1", "true")
+
+
 def record_traffic(csv_path, workload):
     """profiles/traffic.json entries of workload's forward passes: DRAM bytes
     read + written per launch, averaged over the captured launches of each
@@ -408,7 +419,7 @@ def record_traffic(csv_path, workload):
         elif "k_kick_pass_c" in name: slot = "kick_c"
         elif "k_kick6" in name: slot = "kick6"
         elif "k_drift_yz" in name: slot = "drift_yz"
-        elif "k_drift_fast" in name and name.split("k_drift_fast<")[1].split(">")[0].split(",")[-1].strip() == "1":
+        elif "k_drift_fast" in name and _drift_with_density(name):
             slot = "drift_x"
         elif "k_drift_fast" in name:
             slot = ("drift_z", "drift_y")[zy % 2]
