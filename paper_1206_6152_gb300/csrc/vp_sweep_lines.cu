@@ -461,14 +461,15 @@ __global__ void __launch_bounds__(Planes<N>::NT, Planes<N>::CTAS) k_kick_planes(
 // CTAs of 128 threads, one line per thread at a time: as many as there are
 // lines for, or with persistent only those that fit on the GPU at once.  The
 // persistent grid pays where every CTA ends with a merge of its losses (FP64
-// kicks of 20 x 18 x 22 cubes 1.14 -> 0.83 ms).
+// kicks of 20 x 18 x 22 cubes 1.14 -> 0.83 ms).  More CTAs than a grid holds (over a
+// terabyte of f) are an error: kernels launched without persistent take one line each.
 template <class K>
 cudaError_t lines_grid(K kernel, long long lines, bool persistent, unsigned &grid)
 {
     const long long g = (lines + 127) / 128;
-    if (!persistent && g <= 0x7fffffffLL) {
+    if (!persistent) {
         grid = (unsigned)g;
-        return cudaSuccess;
+        return g <= 0x7fffffffLL ? cudaSuccess : cudaErrorInvalidConfiguration;
     }
     int per_sm = 0;
     const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 128, 0);
