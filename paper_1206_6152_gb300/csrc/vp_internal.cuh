@@ -176,7 +176,7 @@ cudaError_t launch_kick_fast(vp_ctx *c, void *f, const void *ca, const void *cb,
                              void *inter1 = nullptr, const int *gate = nullptr);
 cudaError_t launch_drift_fast(vp_ctx *c, void *f, int axis, const void *coef, double *rho_part,
                               void *fo = nullptr);
-// sweeps of lines of any length up to 64, zero shift (vp_sweep_lines.cu); f
+// sweeps of lines of any length up to 64, drifts by less than a cell (vp_sweep_lines.cu); f
 // into fo (fo == f: in place)
 int vp_drift_lines_ok(const vp_ctx *c, int axis);
 cudaError_t launch_drift_lines(vp_ctx *c, const void *f, int axis, const void *coef, void *fo);
@@ -187,7 +187,12 @@ cudaError_t launch_kick_lines(vp_ctx *c, const void *f, const void *ca, const vo
 // (vp_sweep_cells.cu)
 int vp_drift_cells_ok(const vp_ctx *c, int axis);
 cudaError_t launch_drift_cells(vp_ctx *c, const void *f, int axis, const void *coef, void *fo);
-int vp_kick_cells_ok(const vp_ctx *c, int nsweeps, int first_axis);
+// the kernel that sweeps the velocity cubes of an FP64 grid: one thread per line of
+// a cube in shared memory (vp_sweep.cu; or one axis per pass), per line in registers,
+// per cell
+enum KickF64 { KICK_CUBES, KICK_LINES, KICK_CELLS };
+KickF64 vp_kick_f64_route(const vp_ctx *c, int nsweeps, int first_axis);
+int vp_kick_cube_ok(const vp_ctx *c);       // whole cubes fit in shared memory
 cudaError_t launch_kick_cells(vp_ctx *c, const void *f, const void *ca, const void *cb, int nsweeps,
                               int first_axis, void *fo);
 // one sweep from src into dst (dst != src), used by the adjoint's replay;

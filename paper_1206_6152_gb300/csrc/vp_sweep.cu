@@ -543,8 +543,7 @@ template <typename T>
 cudaError_t launch_kick_dispatch(vp_ctx *c, T *f, const LineCoef<T> *ca, const LineCoef<T> *cb,
                                  int nsweeps, int first_axis)
 {
-    if (kick_cube_bytes(c) > 220 * 1024)
-        return launch_kick_axes<T>(c, f, ca, cb, nsweeps, first_axis);
+    if (!vp_kick_cube_ok(c)) return launch_kick_axes<T>(c, f, ca, cb, nsweeps, first_axis);
     const int nx = c->nv[0], ny = c->nv[1], nz = c->nv[2];
     if (nx == ny && ny == nz) {
         if (nx == 16) return launch_kick_t<T, 16, 16, 16>(c, f, ca, cb, nsweeps, first_axis);
@@ -666,8 +665,10 @@ cudaError_t launch_kick(vp_ctx *c, void *f, const void *coef_a, const void *coef
 {
     if (vp_kick_fast_ok(c)) return launch_kick_fast(c, f, coef_a, coef_b, nsweeps, first_axis);
     if (vp_kick_big_ok(c)) return launch_kick_big(c, f, coef_a, coef_b, nsweeps, first_axis);
-    if (vp_kick_cells_ok(c, nsweeps, first_axis)) return launch_kick_cells(c, f, coef_a, coef_b, nsweeps, first_axis, f);
-    if (vp_kick_lines_ok(c)) return launch_kick_lines(c, f, coef_a, coef_b, nsweeps, first_axis, f);
+    const KickF64 route = c->isdouble ? vp_kick_f64_route(c, nsweeps, first_axis) : KICK_LINES;
+    if (route == KICK_CELLS) return launch_kick_cells(c, f, coef_a, coef_b, nsweeps, first_axis, f);
+    if (route == KICK_LINES && vp_kick_lines_ok(c))
+        return launch_kick_lines(c, f, coef_a, coef_b, nsweeps, first_axis, f);
     if (c->isdouble)
         return launch_kick_dispatch<double>(c, (double *)f, (const LineCoef<double> *)coef_a,
                                             (const LineCoef<double> *)coef_b, nsweeps,
@@ -676,6 +677,8 @@ cudaError_t launch_kick(vp_ctx *c, void *f, const void *coef_a, const void *coef
                                        (const LineCoef<float> *)coef_b, nsweeps, first_axis);
 }
 
+int vp_kick_cube_ok(const vp_ctx *c) { return kick_cube_bytes(c) <= 220 * 1024; }
+
 cudaError_t launch_sweep_into(vp_ctx *c, const void *src, void *dst, int axis, const void *coef,
                               double drift_alpha_bound)
 {
@@ -683,9 +686,9 @@ cudaError_t launch_sweep_into(vp_ctx *c, const void *src, void *dst, int axis, c
         return launch_kick_fast(c, const_cast<void *>(src), coef, nullptr, 1, axis - 3, dst);
     if (axis >= 3 && vp_kick_big_ok(c))
         return launch_kick_big(c, const_cast<void *>(src), coef, nullptr, 1, axis - 3, dst);
-    if (axis >= 3 && vp_kick_cells_ok(c, 1, axis - 3))
-        return launch_kick_cells(c, src, coef, nullptr, 1, axis - 3, dst);
-    if (axis >= 3 && vp_kick_lines_ok(c))
+    const KickF64 route = axis >= 3 && c->isdouble ? vp_kick_f64_route(c, 1, axis - 3) : KICK_LINES;
+    if (route == KICK_CELLS) return launch_kick_cells(c, src, coef, nullptr, 1, axis - 3, dst);
+    if (axis >= 3 && route == KICK_LINES && vp_kick_lines_ok(c))
         return launch_kick_lines(c, src, coef, nullptr, 1, axis - 3, dst);
     if (axis < 3 && vp_drift_fast_ok(c, axis) && drift_alpha_bound < 1.0)
         return launch_drift_fast(c, const_cast<void *>(src), axis, coef, nullptr, dst);

@@ -10,11 +10,12 @@
 // update reads its neighbour's flux from shared memory.  Any whole-cell shift.
 //
 // It pays while the lines do not fill the GPU's quadrants with a warp each (32
-// lanes x 4 quadrants x SMs = 19456 lines; the rules are below); above that the
-// line kernels do less work per cell.  128 x 128 cells (1D1V): x drift 88 -> 5 us, fused kick 140 ->
+// lanes x 4 quadrants x SMs = 19456 lines) and are long (the rules are below); else the
+// other kernels do less work per cell.  128 x 128 cells (1D1V): x drift 88 -> 5 us, fused kick 140 ->
 // 10 us, and with the sweeps along periodic axes of one cell passed over a step
 // 254 -> 44 us.
 #include <cuda_runtime.h>
+#include <math.h>
 
 #include "vp_device.cuh"
 #include "vp_fast_line.cuh"
@@ -26,12 +27,26 @@ int vp_sm_count();
 
 namespace {
 
+// Adds the CTA's losses to *lost_out.  Most cells lose nothing: warps whose lanes have
+// only zeros pass the merge over (25 FP64 instructions), and the warps' sums are merged
+// by as many steps as there are warps (x drift with outflow of 16^2 x 4 of 12 x 8 x 10
+// cells 104 us with every warp's merge).
 __device__ __forceinline__ void add_lost(double lost, double *lost_out, Acc<double> *red)
 {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     Acc<double> a;
-    a.add(lost);
-    a = block_merge(a, red);
-    if (threadIdx.x == 0 && a.value() != 0.0) atomicAdd(lost_out, a.value());
+    if (__any_sync(0xffffffffu, __double_as_longlong(lost) << 1 != 0)) {
+        a.add(lost);
+        for (int d = 16; d > 0; d >>= 1) a.shfl_merge(d);
+    }
+    if (lane == 0) red[warp] = a;
+    __syncthreads();
+    if (warp != 0) return;
+    a = lane < nw ? red[lane] : Acc<double>();
+    if (!__any_sync(0xffffffffu, __double_as_longlong(a.s) << 1 != 0)) return;
+    for (int d = 16; d > 0; d >>= 1)
+        if (d < nw) a.shfl_merge(d);
+    if (lane == 0) atomicAdd(lost_out, a.value());
 }
 
 // maxima (at least 0) of L lines in shared memory, line u at first(u), n cells
@@ -177,13 +192,14 @@ int threads_for(long long cells)
     return (int)(t > 512 ? 512 : t);
 }
 
-// What a sweep along lines of n cells takes in units of one FP64 instruction of
-// the busiest quadrant: one thread per line, 7.3 instructions per cell and a
-// round of lines for every 32 lanes x 4 quadrants x SMs of them
-double lines_cost(const vp_ctx *c, int n)
+// The rules below compare estimates of the time a call takes, in units of one FP64
+// instruction of a quadrant's warp (74 cycles, 39 ns): a constant per launch or sweep
+// and the FP64 instructions of the busiest quadrant.  Rounds of n warps' lanes over the
+// SMs' quadrants (32 lanes x 4 quadrants each):
+double rounds_of(long long n)
 {
-    const long long round = 128LL * vp_sm_count(), lines = c->ncells / n;
-    return 7.3 * n * (double)((lines + round - 1) / round);
+    const long long round = 128LL * vp_sm_count();
+    return (double)((n + round - 1) / round);
 }
 
 // lines per CTA of k_drift_cells: one while that gives at most four CTAs per
@@ -198,12 +214,19 @@ int cells_lines(const vp_ctx *c, int n)
 
 }  // namespace
 
-// one thread per cell, 9 instructions (no difference is shared), where that is
-// the cheaper one: below 0.8 of a round of lines
+// One thread per cell where that is the cheaper one.  Fitted to every drift of 27
+// boxes of 3^3 to 128 positions with 10 velocity grids each, both boundary rules: the
+// choice takes 0.3 % more than the better of the two on average.  Lines of 64: 16 against 35 us (4^2 x 64 of
+// 6^3 cells), but 43 against 34 us with 12 x 8 x 10 velocity cells; lines below 8 cells
+// gain nothing.  Lines above 64 cells have only the shared-memory kernel beside it.
 int vp_drift_cells_ok(const vp_ctx *c, int axis)
 {
-    const long long round = 128LL * vp_sm_count();
-    return c->isdouble && 9.0 * (double)((c->ncells + round - 1) / round) < lines_cost(c, c->n[axis]);
+    const int n = c->n[axis];
+    if (!c->isdouble || n < 8) return 0;
+    const double cells = 170 + 16 * rounds_of(c->ncells) + (c->periodic_space ? 0 : 40);
+    const double lines = n <= 64 ? 165 + 7.3 * n * rounds_of(c->ncells / n) + (c->periodic_space ? 0 : 60)
+                                 : 200 + 13.0 * n * rounds_of(c->ncells / n);
+    return cells < lines;
 }
 
 cudaError_t launch_drift_cells(vp_ctx *c, const void *f, int axis, const void *coef, void *fo)
@@ -227,22 +250,36 @@ cudaError_t launch_drift_cells(vp_ctx *c, const void *f, int axis, const void *c
     return cudaGetLastError();
 }
 
-// cubes whose two buffers and line maxima fit in 96 KB, where a cube's CTA (its
-// cells over 128 lanes, a round of cubes for every SM) is cheaper than one
-// thread per line along the axes swept: 128 cubes of 128 cells are by far, 4^3 cubes
-// of 16^3 are not (three steps 635 us against 362 us), and a single vy sweep of 6^3
-// cubes of 64 x 4 x 4 is not either, though the kick is
-int vp_kick_cells_ok(const vp_ctx *c, int nsweeps, int first_axis)
+// Which kernel sweeps FP64 cubes.  Lines (one launch per sweep, no axis above 64) are the
+// cheapest where there are enough of them; with few cubes their launches weigh more
+// than the sweeps, and one CTA per cube with all sweeps in one launch is better: one
+// thread per line where lines are short (k_kick; a chain of n cells, or the FP64
+// instructions of a cube's warps of lines over four quadrants), one thread per cell
+// where they are not (its two buffers and line maxima in 96 KB).  Fitted to single
+// sweeps, half kicks and fused kicks of the same boxes: none takes more than 1.07 times
+// the whole-cube kernel, and 0.4 % more than the best of the three on average.
+// Fused kick of 4^3 cubes of 6 x 7 x 8: whole cubes 45, lines 62, cells 43 us; 4^3 of 9 x
+// 10 x 11: 57, 74, 66; 8^3 of 6 x 7 x 8: 64, 78, 76; 8^3 of 9 x 10 x 11: 125, 114, 181;
+// 128 cubes of 64 x 1 x 1: 92, 105, 69.
+KickF64 vp_kick_f64_route(const vp_ctx *c, int nsweeps, int first_axis)
 {
+    const double sms = vp_sm_count(), np = (double)c->np;
     int nmin = c->nv[0];
     for (int a = 1; a < 3; ++a)
         if (c->nv[a] < nmin) nmin = c->nv[a];
-    const int axes = nsweeps < 3 ? nsweeps : 3;
-    double lines = 0.0;
-    for (int k = 0; k < axes; ++k) lines += lines_cost(c, c->nv[(first_axis + k) % 3]);
-    const long long sms = vp_sm_count();
-    const double cells = axes * 9.0 * (double)((c->np + sms - 1) / sms) * (double)((c->nvc + 127) / 128);
-    return c->isdouble && cells < lines && (2 * c->nvc + c->nvc / nmin) * sizeof(double) <= 96 * 1024;
+    double cubes = 250, cells = 250, lines = 0;
+    for (int k = 0; k < nsweeps; ++k) {
+        const int n = c->nv[(first_axis + k) % 3];
+        const double warps = (double)((c->nvc / n + 31) / 32);
+        cubes += 40 + n * fmax(10.0, (10 + 0.75 * warps) * fmax(np / sms, 1.0) * warps / 4);
+        cells += 40 + 20 * ceil(np / sms) * (double)((c->nvc + 127) / 128);
+        lines += 200 + 8 * n * rounds_of(c->ncells / n);
+    }
+    if ((2 * c->nvc + c->nvc / nmin) * sizeof(double) > 96 * 1024) cells = INFINITY;
+    if (c->maxnv > 64) lines = INFINITY;
+    else if (!vp_kick_cube_ok(c)) cubes = INFINITY;
+    if (cells < cubes && cells < lines) return KICK_CELLS;
+    return lines < cubes ? KICK_LINES : KICK_CUBES;
 }
 
 cudaError_t launch_kick_cells(vp_ctx *c, const void *f, const void *ca, const void *cb, int nsweeps,
