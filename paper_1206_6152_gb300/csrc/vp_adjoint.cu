@@ -334,50 +334,50 @@ __global__ void __launch_bounds__(256) k_functional_grad(T *__restrict__ lam_f,
 
 // ---------------------------------------------------------------------------
 // FP32 register-line adjoint (line lengths 16/32/48/64, zero whole-cell shift;
-// other lengths and FP64: vp_adjoint_lines.cu): the line of f, the output cotangent and the input cotangent live in
-// registers; the arms are evaluated with the same strict comparisons as
-// line_adjoint.  A line with a whole-cell shift is left untouched and
+// other lengths and FP64: vp_adjoint_lines.cu): the line of f, the output cotangent
+// and the input cotangent live in registers; the arms are evaluated with the same
+// strict comparisons as line_adjoint.  A line with a whole-cell shift is left untouched and
 // flagged for the generic kernel.
 // ---------------------------------------------------------------------------
-template <typename T, int N, bool PERIODIC, bool NEG>
-__device__ __forceinline__ T adjoint_regs(const T (&f)[N], const T (&lo)[N], T (&li)[N],
-                                          const LineCoef<T> &cf)
+template <int N, bool PERIODIC, bool NEG>
+__device__ __forceinline__ float adjoint_regs(const float (&f)[N], const float (&lo)[N], float (&li)[N],
+                                          const LineCoef<float> &cf)
 {
 #define M(j) (NEG ? N - 1 - (j) : (j))
-    const T c0 = cf.c0, c1 = cf.c1, c2 = cf.c2;
-    const T beta = c0;
-    const T dc1 = (T(2) - T(6) * beta + T(3) * beta * beta) / T(6);
-    const T dc2 = (T(1) - T(3) * beta * beta) / T(6);
-    T finf = T(0);
+    const float c0 = cf.c0, c1 = cf.c1, c2 = cf.c2;
+    const float beta = c0;
+    const float dc1 = (2.f - 6.f * beta + 3.f * beta * beta) / 6.f;
+    const float dc2 = (1.f - 3.f * beta * beta) / 6.f;
+    float finf = 0.f;
     int arg = 0;
 #pragma unroll
     for (int j = 0; j < N; ++j) {
-        const T v = f[M(j)];
+        const float v = f[M(j)];
         if (v > finf) { finf = v; arg = j; }
     }
 #pragma unroll
     for (int j = 0; j < N; ++j) li[j] = lo[j];
-    T lfinf = T(0), dbeta = T(0);
+    float lfinf = 0.f, dbeta = 0.f;
 #pragma unroll
     for (int j = 0; j < N; ++j) {
-        const T lnext = (j + 1 < N) ? lo[M(j + 1)] : (PERIODIC ? lo[M(0)] : T(0));
-        const T mu = lnext - lo[M(j)];
-        const T fm = (j > 0) ? f[M(j - 1)] : (PERIODIC ? f[M(N - 1)] : T(0));
-        const T f0 = f[M(j)];
-        const T fp = (j + 1 < N) ? f[M(j + 1)] : (PERIODIC ? f[M(0)] : T(0));
-        const T two_f0 = T(2) * f0, two_gap = T(2) * (finf - f0);
-        const T dp = fp - f0, dm = f0 - fm;
-        const bool pu = dp > T(0) && two_f0 < dp;
-        const bool pl = !pu && dp < T(0) && -two_gap > dp;
-        const bool mup = dm > T(0) && two_gap < dm;
-        const bool mlo = !mup && dm < T(0) && -two_f0 > dm;
-        const T ep = pu ? two_f0 : (pl ? -two_gap : dp);
-        const T em = mup ? two_gap : (mlo ? -two_f0 : dm);
-        const T a = c1 * mu, b = c2 * mu;
-        T l0 = c0 * mu;
-        l0 += (pu || pl) ? T(2) * a : -a;
-        l0 += (mup || mlo) ? -T(2) * b : b;
-        lfinf += (pl ? -T(2) * a : T(0)) + (mup ? T(2) * b : T(0));
+        const float lnext = (j + 1 < N) ? lo[M(j + 1)] : (PERIODIC ? lo[M(0)] : 0.f);
+        const float mu = lnext - lo[M(j)];
+        const float fm = (j > 0) ? f[M(j - 1)] : (PERIODIC ? f[M(N - 1)] : 0.f);
+        const float f0 = f[M(j)];
+        const float fp = (j + 1 < N) ? f[M(j + 1)] : (PERIODIC ? f[M(0)] : 0.f);
+        const float two_f0 = 2.f * f0, two_gap = 2.f * (finf - f0);
+        const float dp = fp - f0, dm = f0 - fm;
+        const bool pu = dp > 0.f && two_f0 < dp;
+        const bool pl = !pu && dp < 0.f && -two_gap > dp;
+        const bool mup = dm > 0.f && two_gap < dm;
+        const bool mlo = !mup && dm < 0.f && -two_f0 > dm;
+        const float ep = pu ? two_f0 : (pl ? -two_gap : dp);
+        const float em = mup ? two_gap : (mlo ? -two_f0 : dm);
+        const float a = c1 * mu, b = c2 * mu;
+        float l0 = c0 * mu;
+        l0 += (pu || pl) ? 2.f * a : -a;
+        l0 += (mup || mlo) ? -2.f * b : b;
+        lfinf += (pl ? -2.f * a : 0.f) + (mup ? 2.f * b : 0.f);
         li[M(j)] += l0;
         if (!(pu || pl)) {
             if (j + 1 < N) li[M(j + 1)] += a;
@@ -396,8 +396,8 @@ __device__ __forceinline__ T adjoint_regs(const T (&f)[N], const T (&lo)[N], T (
     return NEG ? -dbeta : dbeta;
 }
 
-template <typename T, int N, bool PERIODIC, bool ROWS>
-__global__ void __launch_bounds__(128) k_adjoint_fast(AdjArgs<T> A, LineGeom g, int *skipped)
+template <int N, bool PERIODIC, bool ROWS>
+__global__ void __launch_bounds__(128) k_adjoint_fast(AdjArgs<float> A, LineGeom g, int *skipped)
 {
     __shared__ double red[32];
     const int t = threadIdx.x;
@@ -407,7 +407,7 @@ __global__ void __launch_bounds__(128) k_adjoint_fast(AdjArgs<T> A, LineGeom g, 
     const long long w = (long long)(vel ? blockIdx.y : blockIdx.x) * blockDim.x + t;
     bool active = w < g.nlines_inner;
     long long base = 0;
-    LineCoef<T> cf;
+    LineCoef<float> cf;
     if (g.axis < 3) {
         const int o = blockIdx.y;
         const long long cell0 = (long long)(o / g.od) * g.m1 + (long long)(o % g.od) * g.m2;
@@ -425,8 +425,8 @@ __global__ void __launch_bounds__(128) k_adjoint_fast(AdjArgs<T> A, LineGeom g, 
     }
     double da = 0.0;
     if (active) {
-        T f[N], lo[N], li[N];
-        if constexpr (ROWS && sizeof(T) == 4) {
+        float f[N], lo[N], li[N];
+        if constexpr (ROWS) {
 #pragma unroll
             for (int j = 0; j < N; j += 4) {
                 const float4 a = *reinterpret_cast<const float4 *>(A.fin + base + j);
@@ -441,10 +441,10 @@ __global__ void __launch_bounds__(128) k_adjoint_fast(AdjArgs<T> A, LineGeom g, 
                 lo[j] = A.lam[base + j * g.stride];
             }
         }
-        const T d = (cf.code & 1) ? adjoint_regs<T, N, PERIODIC, true>(f, lo, li, cf)
-                                  : adjoint_regs<T, N, PERIODIC, false>(f, lo, li, cf);
+        const float d = (cf.code & 1) ? adjoint_regs<N, PERIODIC, true>(f, lo, li, cf)
+                                      : adjoint_regs<N, PERIODIC, false>(f, lo, li, cf);
         da = (double)d;
-        if constexpr (ROWS && sizeof(T) == 4) {
+        if constexpr (ROWS) {
 #pragma unroll
             for (int j = 0; j < N; j += 4)
                 *reinterpret_cast<float4 *>(A.lam + base + j) =
@@ -466,18 +466,18 @@ int vp_adjoint_fast_ok(const vp_ctx *c, int axis)
     return !c->isdouble && (n == 16 || n == 32 || n == 48 || n == 64);
 }
 
-template <typename T, int N>
-cudaError_t adjoint_fast_n(vp_ctx *c, const AdjArgs<T> &A, const LineGeom &g, dim3 grid)
+template <int N>
+cudaError_t adjoint_fast_n(vp_ctx *c, const AdjArgs<float> &A, const LineGeom &g, dim3 grid)
 // grid: (line chunks, outer index or cube)
 {
-    const bool rows = g.stride == 1 && sizeof(T) == 4 && (c->nvc % 4) == 0;
+    const bool rows = g.stride == 1 && (c->nvc % 4) == 0;
     if (g.axis >= 3) grid = dim3(grid.y, grid.x);        // (cube, chunk)
     if (A.periodic) {
-        if (rows) k_adjoint_fast<T, N, true, true><<<grid, 128, 0, c->stream>>>(A, g, c->adj_flag);
-        else k_adjoint_fast<T, N, true, false><<<grid, 128, 0, c->stream>>>(A, g, c->adj_flag);
+        if (rows) k_adjoint_fast<N, true, true><<<grid, 128, 0, c->stream>>>(A, g, c->adj_flag);
+        else k_adjoint_fast<N, true, false><<<grid, 128, 0, c->stream>>>(A, g, c->adj_flag);
     } else {
-        if (rows) k_adjoint_fast<T, N, false, true><<<grid, 128, 0, c->stream>>>(A, g, c->adj_flag);
-        else k_adjoint_fast<T, N, false, false><<<grid, 128, 0, c->stream>>>(A, g, c->adj_flag);
+        if (rows) k_adjoint_fast<N, false, true><<<grid, 128, 0, c->stream>>>(A, g, c->adj_flag);
+        else k_adjoint_fast<N, false, false><<<grid, 128, 0, c->stream>>>(A, g, c->adj_flag);
     }
     return cudaGetLastError();
 }
@@ -487,10 +487,10 @@ cudaError_t launch_adjoint_fast(vp_ctx *c, const AdjArgs<float> &A, const LineGe
     cudaError_t e = cudaMemsetAsync(c->adj_flag, 0, sizeof(int), c->stream);
     if (e != cudaSuccess) return e;
     switch (g.n) {
-    case 16: return adjoint_fast_n<float, 16>(c, A, g, grid);
-    case 32: return adjoint_fast_n<float, 32>(c, A, g, grid);
-    case 48: return adjoint_fast_n<float, 48>(c, A, g, grid);
-    default: return adjoint_fast_n<float, 64>(c, A, g, grid);
+    case 16: return adjoint_fast_n<16>(c, A, g, grid);
+    case 32: return adjoint_fast_n<32>(c, A, g, grid);
+    case 48: return adjoint_fast_n<48>(c, A, g, grid);
+    default: return adjoint_fast_n<64>(c, A, g, grid);
     }
 }
 

@@ -170,18 +170,17 @@ __global__ void __launch_bounds__(256) k_kick_plane(T *__restrict__ f,
 }
 
 // ---------------------------------------------------------------------------
-// kick: NX, NY, NZ compile-time cube edges (0 = runtime)
+// kick of whole cubes in shared memory
 // ---------------------------------------------------------------------------
-template <typename T, int NX, int NY, int NZ>
+template <typename T>
 __global__ void __launch_bounds__(1024) k_kick(T *__restrict__ f, const LineCoef<T> *__restrict__ ca,
                                                const LineCoef<T> *__restrict__ cb, int nsweeps,
-                                               int first_axis, int rnx, int rny, int rnz,
+                                               int first_axis, int nx, int ny, int nz,
                                                long long np, double *lost_out)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *cube = reinterpret_cast<T *>(smem_raw);
     __shared__ Acc<double> red[32];
-    const int nx = NX ? NX : rnx, ny = NY ? NY : rny, nz = NZ ? NZ : rnz;
     const int P = nz | 1;                      // odd row pitch
     const int ncube = nx * ny * nz;
     T lost = T(0);
@@ -461,8 +460,8 @@ int sm_count()
     return n;
 }
 
-template <typename T, int NX, int NY, int NZ>
-cudaError_t launch_kick_t(vp_ctx *c, T *f, const LineCoef<T> *ca, const LineCoef<T> *cb,
+template <typename T>
+cudaError_t launch_kick_cubes(vp_ctx *c, T *f, const LineCoef<T> *ca, const LineCoef<T> *cb,
                           int nsweeps, int first_axis)
 {
     const int nx = c->nv[0], ny = c->nv[1], nz = c->nv[2];
@@ -474,7 +473,7 @@ cudaError_t launch_kick_t(vp_ctx *c, T *f, const LineCoef<T> *ca, const LineCoef
     int threads = ((lines + 31) / 32) * 32;
     if (threads > 1024) threads = 1024;
     if (threads < 64) threads = 64;
-    auto kern = k_kick<T, NX, NY, NZ>;
+    auto kern = k_kick<T>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
@@ -544,12 +543,7 @@ cudaError_t launch_kick_dispatch(vp_ctx *c, T *f, const LineCoef<T> *ca, const L
                                  int nsweeps, int first_axis)
 {
     if (!vp_kick_cube_ok(c)) return launch_kick_axes<T>(c, f, ca, cb, nsweeps, first_axis);
-    const int nx = c->nv[0], ny = c->nv[1], nz = c->nv[2];
-    if (nx == ny && ny == nz) {
-        if (nx == 16) return launch_kick_t<T, 16, 16, 16>(c, f, ca, cb, nsweeps, first_axis);
-        if (nx == 32) return launch_kick_t<T, 32, 32, 32>(c, f, ca, cb, nsweeps, first_axis);
-    }
-    return launch_kick_t<T, 0, 0, 0>(c, f, ca, cb, nsweeps, first_axis);
+    return launch_kick_cubes<T>(c, f, ca, cb, nsweeps, first_axis);
 }
 
 template <typename T>
