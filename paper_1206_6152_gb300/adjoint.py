@@ -84,7 +84,7 @@ class _Trajectory(torch.autograd.Function):
         sim: VlasovPoisson = ctx.sim
         f = sim.f
         fbytes = f.numel() * f.element_size()
-        # the adjoint's scratch states (nine at most) are allocated by the library,
+        # the adjoint's scratch states (eight at most) are allocated by the library,
         # outside torch's caching allocator: blocks torch keeps cached would not be
         # available to it, and go back to the device where it might run short
         if f.is_cuda and _free_bytes(f.device) < (ctx.every + 16) * fbytes:

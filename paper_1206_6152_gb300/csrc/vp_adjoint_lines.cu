@@ -16,7 +16,7 @@
 // own slots (a warp copies neighbouring cells); vz rows go through a tile, rows
 // at odd pitch, with the CTA's contiguous rows copied in and out coalesced.
 //
-// What bounds it: FP32 issue and HBM, 12 bytes per cell; FP64 the FP64 pipe (74
+// What bounds it: FP32 issue and HBM, 12 bytes per cell; FP64 the FP64 pipe (64
 // cycles per warp instruction): comparisons, doublings and selections of FP64 run
 // on the integer pipes, which leaves 13 FP64 instructions per cell, 17 with the
 // beta derivative.  Measured, one sweep: FP32 20 x 18 x 22 of 24 x 28 x 26 cells

@@ -8,8 +8,9 @@
 #include "vp_internal.cuh"
 
 // ---------------------------------------------------------------------------
-// FP64 minimum and maximum on the integer pipes: GB300 issues FP64
-// instructions at a small fraction of its integer rate, and a comparison of
+// FP64 minimum and maximum on the integer pipes: an FP64 instruction takes 64 cycles of
+// a quadrant's FP64 pipe per warp, however few lanes are active (measured with the SM's
+// clock counter: 64.0 with one to four warps per quadrant), and a comparison of
 // two doubles is exact on a key of their bits that orders every non-NaN
 // double as its value (-0 below +0).  vmin/vmax: these for double, the FP32
 // instructions for float.
@@ -145,7 +146,7 @@ struct Acc<double> {
     double s = 0.0, c = 0.0;
     // Neumaier's sum with the larger operand chosen by its exponent (that is
     // all the error term needs to be exact) on the integer pipes: four FP64
-    // instructions of 74 pipe cycles each; comparing and subtracting in both
+    // instructions of 64 pipe cycles each; comparing and subtracting in both
     // orders took eight
     __device__ __forceinline__ void add(double x)
     {

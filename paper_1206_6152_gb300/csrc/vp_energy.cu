@@ -5,7 +5,7 @@
 //    and the density with them.  A thread owns columns (vy, vz) and runs along
 //    vx: with M_c = sum_i f and W_c = sum_i f vx_i^2 of a column,
 //    sum f |v|^2 = sum_c W_c + (vy^2 + vz^2)_c M_c.
-//    FP32 f: an FP64 instruction takes 74 cycles of its quadrant's pipe, so the sums
+//    FP32 f: an FP64 instruction takes 64 cycles of its quadrant's pipe, so the sums
 //    are kept on the FP32 pipe as three floats each (TwoSum; products by TwoProd, with
 //    weights of three floats: about 27 FP32 instructions per cell), whose roundings lie
 //    below those of FP64 compensated sums, and turned into FP64 once per cube.  Bound by

@@ -3,8 +3,8 @@
 // other small boxes).
 //
 // With one thread per line a 128-cell line is a serial chain of 128 x 7 FP64
-// instructions of 74 pipe cycles each, on as many quadrants as there are warps
-// of lines: 128 lines of 128 kept four of the GPU's 608 quadrants busy for 84 us.
+// instructions of 64 pipe cycles and their latencies, on as many quadrants as there are
+// warps of lines: 128 lines of 128 kept four of the GPU's 608 quadrants busy for 84 us.
 // Here the lines are staged in shared memory, every thread computes the flux of
 // its own cells (pfc_flux, bit for bit the line routines' arithmetic), and the
 // update reads its neighbour's flux from shared memory.  Any whole-cell shift.
@@ -192,9 +192,9 @@ int threads_for(long long cells)
     return (int)(t > 512 ? 512 : t);
 }
 
-// The rules below compare estimates of the time a call takes, in units of one FP64
-// instruction of a quadrant's warp (74 cycles, 39 ns): a constant per launch or sweep
-// and the FP64 instructions of the busiest quadrant.  Rounds of n warps' lanes over the
+// The rules below compare estimates of the time a call takes, in units of 39 ns (an FP64
+// instruction of a quadrant's warp, 64 cycles or 33 ns, with the gaps that these kernels
+// leave): a constant per launch or sweep and the FP64 instructions of the busiest quadrant.  Rounds of n warps' lanes over the
 // SMs' quadrants (32 lanes x 4 quadrants each):
 double rounds_of(long long n)
 {

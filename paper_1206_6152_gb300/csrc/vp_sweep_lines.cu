@@ -12,7 +12,7 @@
 //    hundred instructions each, lines of 4 to 20 cells were bound by issue (x drift
 //    of 4 x 64^2 of 32^3 cells 1.65 -> 1.36 ms, 8 x 8 x 4 of 48^3, z 95 -> 80, x 60 ->
 //    53 us).  FP64: at the FP64 pipe's rate (7.3 instructions per cell counted,
-//    74 cycles each per quadrant's warp); 20 x 18 x 22 of the same 1.48 -> 0.86
+//    64 cycles each per quadrant's warp); 20 x 18 x 22 of the same 1.48 -> 0.86
 //    ms, and FP64 lines of 16 and 32 go through here as well: the saturating
 //    form takes 9 FP64 instructions and a reciprocal per line, and the z drift
 //    ran both directions' code in every warp (16^6: 0.59 -> 0.25 ms).
