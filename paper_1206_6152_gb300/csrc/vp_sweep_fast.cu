@@ -913,10 +913,12 @@ cudaError_t drift_fast_n(vp_ctx *c, float *f, int axis, const LineCoef<float> *c
     if (rho_part) {
         constexpr size_t racc = (size_t)N * 128 * sizeof(Acc<float>);   // density sums
         // lines of more than 32 cells singly, but those of 48 in pairs where a CTA has more
-        // than a hundred turns (48^6, 216 turns: 15.7 ms against 16.4; 48 x 32^2 of 32^3, 43
-        // turns: 2.51 against 2.36)
+        // than 72 turns of 128 pairs.  Measured, single / pairs in ms: 31 turns (50^2 of 20^3)
+        // 1.40 / 1.51, 43 (32^2 of 32^3) 2.36 / 2.51, 54 (50^2 of 24^3) 2.33 / 2.35, 61 (32^2 of 36^3)
+        // 3.22 / 3.32, 83 (32^2 of 40^3) 4.72 / 4.62, 86 (50^2 of 28^3) 3.67 / 3.55, 111 (32^2 of 44^3)
+        // 6.03 / 5.88, 128 (50^2 of 32^3) 5.41 / 5.14, 216 (48 x 40 of 48^3) 13.78 / 13.17
         constexpr bool LONG = N > 32;
-        const bool single = LONG && (N != 48 || g.per_part <= 100 * 128);
+        const bool single = LONG && (N != 48 || g.per_part <= 72 * 128);
         auto kern = c->periodic_space ? k_drift_fast<N, true, LONG, true> : k_drift_fast<N, false, LONG, true>;
         if constexpr (N == 48) {
             if (!single) kern = c->periodic_space ? k_drift_fast<N, true, false, true> : k_drift_fast<N, false, false, true>;
