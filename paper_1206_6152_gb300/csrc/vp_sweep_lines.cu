@@ -30,9 +30,11 @@
 //    cell and sweep, 15 of them the flux and update), so the line loops go in
 //    whole groups of four cells where NMAX fits the lines, and the tile is
 //    addressed as shared memory.  Fused six-sweep kick against the shared-memory
-//    lines of vp_sweep.cu: 24 x 28 x 26 cubes (554 MB of traffic) 1.83 -> 0.93
-//    ms, 24^3 (764 MB) 2.78 -> 1.19 ms, 40^3 (1.0 GB) 5.1 -> 2.4 ms, 64^3 (537
-//    MB) 2.56 -> 1.18 ms.
+//    lines of vp_sweep.cu: 24 x 28 x 26 cubes (553 MB of f) 1.83 -> 0.89 ms, 24^3
+//    (764 MB) 2.77 -> 1.15 ms.
+//  * k_kick_planes: the vy and vz sweeps of cubes too large for that whose vx planes are
+//    40^2, 48^2, 56^2 or 64^2, at compile-time length.  With k_kick_lines along vx, fused
+//    kick: 40^3 (1.05 GB) 5.2 -> 1.76 ms, 64^3 (537 MB) 2.53 -> 0.84 ms.
 #include <cuda_runtime.h>
 
 #include "vp_clamp_line.cuh"
