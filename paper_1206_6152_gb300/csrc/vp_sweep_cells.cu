@@ -257,7 +257,8 @@ cudaError_t launch_drift_cells(vp_ctx *c, const void *f, int axis, const void *c
 // instructions of a cube's warps of lines over four quadrants), one thread per cell
 // where they are not (its two buffers and line maxima in 96 KB).  Fitted to single
 // sweeps, half kicks and fused kicks of the same boxes: none takes more than 1.07 times
-// the whole-cube kernel, and 0.4 % more than the best of the three on average.
+// the whole-cube kernel (150 x 2 of 12^3, not among them, 1.14), and 0.4 % more than the
+// best of the three on average.
 // Fused kick of 4^3 cubes of 6 x 7 x 8: whole cubes 45, lines 62, cells 43 us; 4^3 of 9 x
 // 10 x 11: 57, 74, 66; 8^3 of 6 x 7 x 8: 64, 78, 76; 8^3 of 9 x 10 x 11: 125, 114, 181;
 // 128 cubes of 64 x 1 x 1: 92, 105, 69.
